@@ -8,13 +8,15 @@
 // looper at the end of its reach), the propagation Jacobian grows like
 // 1/cos(alpha) and the predicted covariance gains a large, nearly rank-one
 // term that the update then removes again; FP32 loses the posterior there.
-// A first FP32 pass fits every track and flags a track as soon as one of its
-// crossings has cos(alpha) below CAREFUL_COS; a second pass refits only the
-// flagged tracks, running those steps' propagation and update in double
+// A first FP32 pass fits every track and stops a track at the first of its
+// crossings with cos(alpha) below CAREFUL_COS; a second pass takes the listed
+// tracks on from there, running such steps' propagation and update in double
 // precision (a small fraction of tracks: loopers near their maximum radius).
 // On a detector with endcap disks, a plane step along more than half a
 // radian of the helix (a looper reaching a disk) flags its track the same
 // way (PLANE_CAREFUL_PSI).
+#include <algorithm>
+
 #include "kf_internal.h"
 
 namespace kfg {
@@ -23,6 +25,7 @@ namespace {
 
 constexpr float CAREFUL_COS = 0.5f;
 constexpr int FIT_THREADS = 128;  // threads per block of the FP32 pass
+constexpr int CAREFUL_BLOCKS = 608;  // careful pass: four warps per SM
 
 // One Kalman step on an endcap disk in scalar type T (the plane, the (r-phi, r)
 // measurement, the disk's scattering and loss).
@@ -133,6 +136,20 @@ __global__ void __launch_bounds__(ORDER_THREADS) k_fit_order(const FitParams P) 
   }
 }
 
+// A track the FP32 pass leaves to the careful pass at step k: the state before
+// that step, the chi2 so far and k wait in the track's own output places.
+__device__ __forceinline__ void leave_to_careful(const FitParams& P, int i, int t, int k, const float (&p)[6],
+                                                 const float (&C)[21], float chi2) {
+#pragma unroll
+  for (int q = 0; q < 6; ++q) P.fit_p[(size_t)q * P.ns + t] = p[q];
+#pragma unroll
+  for (int q = 0; q < 21; ++q) P.fit_C[(size_t)q * P.ns + t] = C[q];
+  P.fit_chi2[t] = chi2;
+  P.fit_status[t] = k;
+  P.careful_list[atomicAdd(P.careful_count, 1u)] = i;
+  if (P.careful_flag) P.careful_flag[t] = 1;
+}
+
 // Track at position i of the fit's order; checkpoints go to column i.
 // Returns, in the careful pass, whether a crossing of the track has
 // cos(alpha) < ADJOINT_CAREFUL_COS (its adjoint then needs double steps).
@@ -153,26 +170,30 @@ __device__ __forceinline__ bool fit_track(const FitParams& P, int i, int t) {
     return false;
   }
   const DevGeom& g = P.g;
+  // the prior, or (careful pass) the state the FP32 pass stopped at before step k0
+  const float* const p0 = CAREFUL ? P.fit_p : P.sp;
+  const float* const C0 = CAREFUL ? P.fit_C : P.sc;
   float p[6], C[21];
 #pragma unroll
-  for (int k = 0; k < 6; ++k) p[k] = P.sp[(size_t)k * P.ns + t];
+  for (int k = 0; k < 6; ++k) p[k] = p0[(size_t)k * P.ns + t];
 #pragma unroll
-  for (int k = 0; k < 21; ++k) C[k] = P.sc[(size_t)k * P.ns + t];
-  // a loose prior: the careful pass runs the first steps in double
-  const bool loose = loose_prior(C, g);
+  for (int k = 0; k < 21; ++k) C[k] = C0[(size_t)k * P.ns + t];
+  const int k0 = CAREFUL ? P.fit_status[t] : 0;
+  // a loose prior: the careful pass runs the first steps in double (a track
+  // left at a later step had no loose prior)
+  const bool loose = k0 == 0 && loose_prior(C, g);
   if (!CAREFUL && loose) {
-    P.careful_list[atomicAdd(P.careful_count, 1u)] = i;
-    if (P.careful_flag) P.careful_flag[t] = 1;
+    leave_to_careful(P, i, t, 0, p, C, 0.f);
     return false;
   }
   const int hoff = P.hit_off[P.seed_event[t]];
   const int n = P.n_list[t];
   const int* lst = P.lists + (size_t)t * P.max_len;
-  float chi2 = 0.f;
+  float chi2 = CAREFUL ? P.fit_chi2[t] : 0.f;
   int status = KF_FIT_OK;
   bool adj_dbl = false;
 #pragma unroll 1
-  for (int k = 0; k < n && status == KF_FIT_OK; ++k) {
+  for (int k = k0; k < n && status == KF_FIT_OK; ++k) {
     if (P.ckpt && k % P.ckpt_stride == 0 && k / P.ckpt_stride < P.ckpt_slices) {  // state before hit k
       float* c = P.ckpt + (size_t)(k / P.ckpt_stride) * 27 * P.ns + i;
 #pragma unroll
@@ -193,23 +214,24 @@ __device__ __forceinline__ bool fit_track(const FitParams& P, int i, int t) {
     }
     if (!CAREFUL && disk) {
       if (k > 0 && plane_careful(g, p, plane_z(g, L))) {  // a long arc onto the disk: the careful pass
-        P.careful_list[atomicAdd(P.careful_count, 1u)] = i;
-        if (P.careful_flag) P.careful_flag[t] = 1;
+        leave_to_careful(P, i, t, k, p, C, chi2);
         return false;
       }
       status = disk_step<float>(g, p, C, k == 0, k + 1 == n, L, mx, my, chi2);
     } else if (!CAREFUL) {
       if (k > 0) {
-        float cosa = 1.f;
-        if (propagate<float, true>(p, C, g.radius[L], field_kb<float>(g, p), INFINITY, &cosa) != 1) {
+        float q[6], J[6][6], cosa = 1.f;
+        if (prop_jacobian<float, true>(p, g.radius[L], field_kb<float>(g, p), INFINITY, q, J, &cosa) != 1) {
           status = KF_FIT_NO_CROSS;
           break;
         }
-        if (cosa < CAREFUL_COS) {  // leave the track to the careful pass
-          P.careful_list[atomicAdd(P.careful_count, 1u)] = i;
-          if (P.careful_flag) P.careful_flag[t] = 1;
+        if (cosa < CAREFUL_COS) {
+          leave_to_careful(P, i, t, k, p, C, chi2);
           return false;
         }
+        transport<float>(J, C);
+#pragma unroll
+        for (int q_ = 0; q_ < 6; ++q_) p[q_] = q[q_];
       }
       Frame f;
       make_frame<float>(p, C, g.vr, g.vz, f);
@@ -252,13 +274,21 @@ __global__ void __launch_bounds__(FIT_THREADS) k_fit(const FitParams P) {
   if (i < P.ns) fit_track<false, DISK>(P, i, P.order[i]);
 }
 
-// Second pass over the flagged tracks (grid-stride over their list).  A
-// track whose adjoint needs double steps gets CAREFUL_DBL_BIT in its entry
-// and is listed in dbl_list.
+// Second pass over the flagged tracks, one warp per block.  Its double steps
+// are bound by the SM's FP64 rate (about 2 FMA per clock and SM, whatever the
+// number of active lanes) and by the divergence of a warp's tracks, so the
+// list is dealt evenly to the blocks: with fewer tracks than blocks, one track
+// per warp.  Taken on from the FP32 pass's last state (one to three steps a
+// track instead of all of them), the fit of 180,000 tracks of 30 events
+// (loads included) went from 551 to 426 us, that of one 2,500-track event
+// with its finding from 825 to 716 us.  A track whose adjoint needs double steps gets CAREFUL_DBL_BIT in
+// its entry and is listed in dbl_list.
 template <bool DISK>
-__global__ void __launch_bounds__(128) k_fit_careful(const FitParams P) {
+__global__ void __launch_bounds__(32) k_fit_careful(const FitParams P) {
   const unsigned n = *P.careful_count;
-  for (unsigned j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+  const unsigned per = min(32u, (n + gridDim.x - 1) / gridDim.x);  // tracks per warp and round
+  if (threadIdx.x >= per) return;
+  for (unsigned j = blockIdx.x * per + threadIdx.x; j < n; j += gridDim.x * per) {
     const unsigned v = (unsigned)P.careful_list[j];
     const int pos = (int)(v & ~CAREFUL_DBL_BIT);
     const bool dbl = fit_track<true, DISK>(P, pos, P.order[pos]);
@@ -299,12 +329,11 @@ cudaError_t launch_fit_main(const FitParams& P, cudaStream_t st) {
 
 cudaError_t launch_fit_careful(const FitParams& P, cudaStream_t st) {
   if (P.ns <= 0) return cudaSuccess;
-  // flagged tracks are a few percent of all, and their double-precision
-  // steps are bound by the SM's FP64 rate: blocks of 32 threads, so that they
-  // spread over many SMs; a grid for a twentieth of all tracks, striding over
-  // however many there are
+  // flagged tracks are a few percent of all: a grid for a twentieth of them
+  // at 32 per block, at least CAREFUL_BLOCKS blocks (of a single track each
+  // in a small batch), striding over however many there are
   const int threads = 32;
-  const int careful_blocks = (P.ns / 20 + threads - 1) / threads + 1;
+  const int careful_blocks = std::max((P.ns / 20 + threads - 1) / threads + 1, std::min(P.ns, CAREFUL_BLOCKS));
   cudaError_t e = cudaMemsetAsync(P.dbl_count, 0, sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
   if (P.g.n_disks > 0) k_fit_careful<true><<<careful_blocks, threads, 0, st>>>(P);
