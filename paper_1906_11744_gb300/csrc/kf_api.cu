@@ -40,7 +40,7 @@ struct kf_ctx {
   DevBuf out_hits, out_n, out_chi2, out_p, out_C, keep, queue, counters, status, tangent, seed_order, check;
   DevBuf sfit, sflag, skeys, x0map;
   // duplicate removal scratch (the conflict lists also serve seed cleaning)
-  DevBuf dd_hit_cnt, dd_owners, dd_conf, dd_nconf, dd_state, dd_scan_tmp;
+  DevBuf dd_head, dd_next, dd_conf, dd_nconf, dd_state;
   // seed cleaning
   DevBuf sc_kin, sc_seed, clean_order, kept_cnt, sc_list, sc_list_cnt;
   // fit
@@ -365,8 +365,8 @@ static std::vector<DevBuf*> all_bufs(kf_ctx* ctx) {
                     &ctx->sc, &ctx->sh, &ctx->seed_event, &ctx->align_raw, &ctx->align4, &ctx->eta_edges, &ctx->eta_lut, &ctx->hb,
                     &ctx->bin_cnt, &ctx->bin_key, &ctx->bin_rank, &ctx->scan_tmp, &ctx->bin_grouped, &ctx->bin_gtab, &ctx->out_hits,
                     &ctx->out_n, &ctx->out_chi2, &ctx->out_p, &ctx->out_C, &ctx->keep, &ctx->queue, &ctx->tangent, &ctx->seed_order, &ctx->check,
-                    &ctx->counters, &ctx->status, &ctx->dd_hit_cnt, &ctx->dd_owners, &ctx->dd_conf,
-                    &ctx->dd_nconf, &ctx->dd_state, &ctx->dd_scan_tmp, &ctx->given_lists, &ctx->given_n, &ctx->fit_p,
+                    &ctx->counters, &ctx->status, &ctx->dd_head, &ctx->dd_next, &ctx->dd_conf,
+                    &ctx->dd_nconf, &ctx->dd_state, &ctx->given_lists, &ctx->given_n, &ctx->fit_p,
                     &ctx->fit_C, &ctx->fit_chi2, &ctx->fit_status, &ctx->careful_list,
                     &ctx->careful_count, &ctx->adj_align_acc, &ctx->adj_align, &ctx->adj_hits,
                     &ctx->adj_seed, &ctx->careful_flag, &ctx->ckpt, &ctx->sc_kin, &ctx->sc_seed,
@@ -416,8 +416,7 @@ int kf_load_hits(kf_ctx* ctx, int n_events, const int* ev_offsets, const float* 
   CK(grow(ctx->scan_tmp, sizeof(unsigned) * scan_tmp_elems(n_bins)));
   CK(grow(ctx->bin_grouped, sizeof(float4) * n));
   CK(grow(ctx->bin_gtab, sizeof(unsigned) * bin_group_elems(n_events, ctx->g.n_surf, ctx->g.n_eta, ctx->g.n_phi)));
-  CK(grow(ctx->dd_hit_cnt, sizeof(unsigned) * ((size_t)n + n_events + 1)));
-  CK(grow(ctx->dd_scan_tmp, sizeof(unsigned) * scan_tmp_elems((size_t)n + n_events)));
+  CK(grow(ctx->dd_head, sizeof(unsigned) * ((size_t)n + n_events)));
   CK(put(ctx->hx.p, x, sizeof(float) * n, device_ptrs, st));
   CK(put(ctx->hy.p, y, sizeof(float) * n, device_ptrs, st));
   CK(put(ctx->hz.p, z, sizeof(float) * n, device_ptrs, st));
@@ -483,7 +482,7 @@ int kf_load_seeds(kf_ctx* ctx, int n_events, const int* ev_offsets, const float*
   CK(grow(ctx->out_p, sizeof(float) * 6 * (size_t)n));
   CK(grow(ctx->out_C, sizeof(float) * 21 * (size_t)n));
   CK(grow(ctx->keep, (size_t)n));
-  CK(grow(ctx->dd_owners, sizeof(int) * (size_t)n * L));
+  CK(grow(ctx->dd_next, sizeof(unsigned) * (size_t)n * L));
   CK(grow(ctx->dd_conf, sizeof(int) * (size_t)n * DEDUP_CONF_CAP));
   CK(grow(ctx->dd_nconf, sizeof(int) * (size_t)n));
   CK(grow(ctx->dd_state, (size_t)n));
@@ -775,9 +774,8 @@ int kf_remove_duplicates(kf_ctx* ctx, void* stream) {
   D.L = ctx->g.n_surf;
   D.ns = ctx->n_seeds;
   D.frac = ctx->cfg.dup_shared_frac;
-  D.e_begin = 0;
-  D.hit_cnt = ptr<unsigned>(ctx->dd_hit_cnt);
-  D.owners = ptr<int>(ctx->dd_owners);
+  D.head = ptr<unsigned>(ctx->dd_head);
+  D.next = ptr<unsigned>(ctx->dd_next);
   D.conf = ptr<int>(ctx->dd_conf);
   D.n_conf = ptr<int>(ctx->dd_nconf);
   D.state = ptr<unsigned char>(ctx->dd_state);
@@ -793,14 +791,12 @@ int kf_remove_duplicates(kf_ctx* ctx, void* stream) {
   }
   if (!ctx->per_event) {
     stage_mark(ctx, 4, st);
-    CK(launch_dedup_batched(D, ctx->n_events, ctx->n_hits, ptr<unsigned>(ctx->dd_scan_tmp),
-                            ctx->dd_scan_tmp.bytes / sizeof(unsigned), st));
+    CK(launch_dedup(D, 0, ctx->n_seeds, 0, ctx->n_events, 0, (size_t)ctx->n_hits + ctx->n_events, st));
     stage_mark(ctx, 5, st);
   } else {
-    for (int e = 0; e < ctx->n_events; ++e) {
-      D.e_begin = e;
-      CK(launch_dedup(D, 1, st));
-    }
+    for (int e = 0; e < ctx->n_events; ++e)
+      CK(launch_dedup(D, ctx->seed_off_h[e], ctx->seed_off_h[e + 1], e, 1, (size_t)ctx->hit_off_h[e] + e,
+                      (size_t)(ctx->hit_off_h[e + 1] - ctx->hit_off_h[e]), st));
   }
   ctx->deduped = true;
   return KF_OK;

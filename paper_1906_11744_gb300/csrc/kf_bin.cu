@@ -346,8 +346,8 @@ __global__ void __launch_bounds__(CELL_THREADS) k_cells(const BinParams P, int e
 size_t scan_tmp_elems(size_t n) { return (n + SCAN_TILE - 1) / SCAN_TILE + 1; }
 
 // Exclusive scan of cnt[0..n) in place plus `add`; cnt[n] = total + add.
-cudaError_t scan_exclusive_inplace(unsigned* cnt, size_t n, unsigned add, unsigned* tmp, size_t tmp_elems,
-                                   cudaStream_t st) {
+static cudaError_t scan_exclusive_inplace(unsigned* cnt, size_t n, unsigned add, unsigned* tmp, size_t tmp_elems,
+                                          cudaStream_t st) {
   const int n_tiles = (int)((n + SCAN_TILE - 1) / SCAN_TILE);
   if ((size_t)n_tiles + 1 > tmp_elems) return cudaErrorInvalidValue;
   k_scan_reduce<<<n_tiles, SCAN_THREADS, 0, st>>>(cnt, n, tmp);

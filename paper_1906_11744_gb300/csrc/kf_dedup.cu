@@ -20,22 +20,27 @@
 // conflict lists and resolution rounds as below, the pairs found by scanning
 // each seed's neighbours in the theta order of the event.
 //
-// Parallel form, identical result:
-//   1. hit -> owning tracks table (count, exclusive scan, fill);
-//   2. for every track, the shared-hit counts with every other track through
-//      that table; a pair over the threshold is a conflict, recorded at the
-//      lower-priority track;
-//   3. resolution rounds: an undecided track is removed as soon as one of its
-//      higher-priority conflicts is kept, and kept as soon as all of them are
-//      removed.  The decisions equal the sequential walk's, because each one
-//      only depends on the final decisions of higher-priority tracks; every
-//      round settles at least the highest-priority undecided track.
-// Batched launch: steps 1-2 one thread per track over the whole batch (the
-// scan over every event's table at once), step 3 one block per event.
-// Single-event launch (per-event form, allocation-free entry): all three
-// steps in one block.
-// Scratch (the owner table, the conflict lists and the decision states) lives
-// in global memory owned by the caller.
+// Parallel form, identical result, over a whole batch or one event:
+//   1. k_dd_build: one thread per hit of a track pushes its entry on the list
+//      of its hit (head[hit] and next[entry], one atomic exchange each);
+//   2. k_dd_conflicts: eight lanes per track test which of its hits have other
+//      owners (for most tracks none: one head and one next read per hit); one
+//      lane walks the lists of those that have and counts the shared hits per
+//      partner; a pair over the threshold is a conflict, recorded at the
+//      lower-priority track; a track without conflicts is kept at once;
+//   3. k_dd_rounds, one block per event: an undecided track is removed as soon
+//      as one of its higher-priority conflicts is kept, and kept as soon as
+//      all of them are removed.  The decisions equal the sequential walk's,
+//      because each one only depends on the final decisions of higher-priority
+//      tracks; every round settles at least the highest-priority undecided
+//      track.
+// All three are bound by the latency and number of the scattered 4-byte
+// accesses to the hit table; lists need one per entry, where a table of owner
+// ranges (count, scan over all hits, fill) needed two and the scan.
+// Measured on an 8,800-track event through the allocation-free entry: 640 us
+// in one block over owner ranges, 46 us so.
+// Scratch (the lists, the conflict lists and the decision states) lives in
+// global memory owned by the caller.
 #include <mutex>
 
 #include "kf_internal.h"
@@ -45,6 +50,9 @@ namespace kfg {
 namespace {
 
 constexpr int DEDUP_THREADS = 1024;
+constexpr int DD_THREADS = 256;
+constexpr int DD_LANES = 8;  // lanes per track when its hits are tested for other owners
+constexpr unsigned DD_NONE = 0xFFFFFFFFu;
 
 // (eta, phi0, |q/pT|) of a state.  phi0 = atan2(-v_x, v_y) with
 // v = h c = (h x - sin phi, h y + cos phi), h times the centre c of the track
@@ -88,40 +96,61 @@ __device__ __forceinline__ bool prio_less(int na, float ca, int ia, int nb, floa
   return ia < ib;
 }
 
-// Owner-table count and fill of track t; cnt is its event's table.
-__device__ __forceinline__ void dd_count(const DedupParams& P, int t, unsigned* cnt) {
-  const int n = P.out_n[t];
-  const int* ht = P.out_hits + (size_t)t * P.L;
-  for (int j = 0; j < n; ++j) atomicAdd(&cnt[ht[j]], 1u);
-}
-__device__ __forceinline__ void dd_fill(const DedupParams& P, int t, unsigned* cnt, int* owners) {
-  const int n = P.out_n[t];
-  const int* ht = P.out_hits + (size_t)t * P.L;
-  for (int j = 0; j < n; ++j) owners[atomicAdd(&cnt[ht[j]], 1u)] = t;
+// Head of the owner list of hit 0 of track t's event (hit h's head at [h]).
+__device__ __forceinline__ unsigned* dd_heads(const DedupParams& P, int t) {
+  if (!P.seed_event) return P.head;  // a single event
+  const int e = P.seed_event[t];
+  return P.head + P.hit_off[e] + e;
 }
 
-// Conflicts of track t (after the fill, hit h's owners are
-// owners[start(h), cnt[h]) with start(h) = cnt[h - 1], start(0) = start0);
-// resets its decision state.
-__device__ __forceinline__ void dd_conflicts(const DedupParams& P, int t, const unsigned* cnt, unsigned start0,
-                                             const int* owners) {
-  const int n = P.out_n[t];
-  if (n == 0) {  // no track (a cleaned seed): removed, nothing to compare
+// Entry id = t L + j for hit j of track t of [t_begin, t_end).
+__global__ void __launch_bounds__(DD_THREADS) k_dd_build(const DedupParams P, int t_begin, int t_end) {
+  const unsigned i = blockIdx.x * (unsigned)DD_THREADS + threadIdx.x;
+  const unsigned r = i / (unsigned)P.L;
+  if (r >= (unsigned)(t_end - t_begin)) return;
+  const int t = t_begin + (int)r, j = (int)(i - r * (unsigned)P.L);
+  if (j >= P.out_n[t]) return;
+  const unsigned id = (unsigned)t * (unsigned)P.L + j;
+  P.next[id] = atomicExch(dd_heads(P, t) + P.out_hits[id], id);
+}
+
+// Conflicts and first decision of the tracks of [t_begin, t_end).
+__global__ void __launch_bounds__(DD_THREADS) k_dd_conflicts(const DedupParams P, int t_begin, int t_end) {
+  const int lane = threadIdx.x & 31, gl = threadIdx.x & (DD_LANES - 1);
+  const int t = t_begin + (int)(blockIdx.x * (DD_THREADS / DD_LANES) + threadIdx.x / DD_LANES);
+  const bool valid = t < t_end;
+  const int L = P.L;
+  const int n = valid ? min(P.out_n[t], L) : 0;
+  const unsigned id0 = (unsigned)t * (unsigned)L;
+  const unsigned* head = valid ? dd_heads(P, t) : P.head;
+  unsigned long long shared = 0;  // bit j: hit j has another entry
+#pragma unroll 3
+  for (int b = 0; b < L; b += DD_LANES) {
+    const int j = b + gl;
+    bool sh = false;
+    if (j < n) {
+      const unsigned nx = P.next[id0 + j];
+      sh = head[P.out_hits[id0 + j]] != id0 + j || nx != DD_NONE;
+    }
+    const unsigned v = __ballot_sync(0xffffffffu, sh);
+    shared |= (unsigned long long)((v >> (lane - gl)) & ((1u << DD_LANES) - 1u)) << b;
+  }
+  if (!valid || gl != 0) return;
+  if (n == 0 || shared == 0) {  // no track (a cleaned seed): removed; nothing shared: kept
     P.n_conf[t] = 0;
-    P.state[t] = 2;
+    P.state[t] = n == 0 ? 2 : 1;
     return;
   }
   const float c = P.out_chi2[t];
-  const int* ht = P.out_hits + (size_t)t * P.L;
   int pid[DEDUP_PARTNER_CAP];
   int pcnt[DEDUP_PARTNER_CAP];
   int np = 0;
   bool overflow = false;
-  for (int j = 0; j < n; ++j) {
-    const int h = ht[j];
-    const unsigned a = h == 0 ? start0 : cnt[h - 1], b = cnt[h];
-    for (unsigned q = a; q < b; ++q) {
-      const int u = owners[q];
+  unsigned long long steps = (unsigned long long)P.ns * L;  // no list is longer
+  for (; shared && !overflow; shared &= shared - 1) {
+    const int j = __ffsll((long long)shared) - 1;
+    for (unsigned q = head[P.out_hits[id0 + j]]; q != DD_NONE && steps; q = P.next[q], --steps) {
+      const int u = (int)(q / (unsigned)L);
       if (u == t) continue;
       int k = 0;
       while (k < np && pid[k] != u) ++k;
@@ -133,6 +162,7 @@ __device__ __forceinline__ void dd_conflicts(const DedupParams& P, int t, const 
         ++np;
       } else {
         overflow = true;
+        break;
       }
     }
   }
@@ -152,7 +182,7 @@ __device__ __forceinline__ void dd_conflicts(const DedupParams& P, int t, const 
     }
   }
   P.n_conf[t] = min(nc, DEDUP_CONF_CAP);
-  P.state[t] = 0;  // undecided
+  P.state[t] = nc == 0 ? 1 : 0;
 }
 
 // Resolution rounds of items [s0, s1) (an event's tracks or seeds) by the
@@ -213,98 +243,10 @@ __device__ void dd_rounds(const Rounds& P, int s0, int s1) {
     for (int t = s0 + threadIdx.x; t < s1; t += blockDim.x) P.keep[t] = P.state[t] == 1 ? 1 : 0;
 }
 
-__global__ void __launch_bounds__(DEDUP_THREADS) k_dedup(const DedupParams P) {
-  __shared__ unsigned sh_scan[33];
-  const int e = P.e_begin + blockIdx.x;
-  const int s0 = P.seed_off[e], s1 = P.seed_off[e + 1];
-  const int h0 = P.hit_off[e], h1 = P.hit_off[e + 1];
-  const int nh = h1 - h0;
-  const int L = P.L;
-  unsigned* cnt = P.hit_cnt + h0 + e;   // nh + 1 entries per event
-  int* owners = P.owners + (size_t)s0 * L;
-  const int tid = threadIdx.x, nt = blockDim.x;
-
-  for (int i = tid; i <= nh; i += nt) cnt[i] = 0u;
-  __syncthreads();
-  for (int t = s0 + tid; t < s1; t += nt) dd_count(P, t, cnt);
-  __syncthreads();
-  // block exclusive scan of cnt[0..nh)
-  {
-    const int per = (nh + nt - 1) / nt;
-    const int b = tid * per;
-    unsigned s = 0;
-    for (int k = 0; k < per; ++k)
-      if (b + k < nh) s += cnt[b + k];
-    // inline block scan
-    const int lane = tid & 31, warp = tid >> 5;
-    unsigned incl = s;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned v = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += v;
-    }
-    if (lane == 31) sh_scan[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-      const int nw = nt >> 5;
-      unsigned w = lane < nw ? sh_scan[lane] : 0u, wi = w;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned v = __shfl_up_sync(0xffffffffu, wi, o);
-        if (lane >= o) wi += v;
-      }
-      if (lane < nw) sh_scan[lane] = wi - w;
-    }
-    __syncthreads();
-    unsigned run = sh_scan[warp] + incl - s;
-    for (int k = 0; k < per; ++k)
-      if (b + k < nh) {
-        const unsigned v = cnt[b + k];
-        cnt[b + k] = run;
-        run += v;
-      }
-  }
-  __syncthreads();
-  // fill: afterwards cnt[h] is the end of hit h's owner range, cnt[h-1] its start
-  for (int t = s0 + tid; t < s1; t += nt) dd_fill(P, t, cnt, owners);
-  __syncthreads();
-  for (int t = s0 + tid; t < s1; t += nt) dd_conflicts(P, t, cnt, 0u, owners);
-  __syncthreads();
-  dd_rounds(Rounds{P.n_conf, P.conf, P.state, P.keep, P.status, ST_DEDUP_ROUNDS, P.max_rounds}, s0, s1);
-}
-
-// Batched steps, one thread per track of the whole batch.  Event e's table
-// is hit_cnt[hit_off[e] + e, hit_off[e + 1] + e] (one extra entry); one
-// exclusive scan over all tables makes the owner positions global.
-__device__ __forceinline__ unsigned* dd_table(const DedupParams& P, int t, int& e) {
-  e = P.seed_event[t];
-  return P.hit_cnt + P.hit_off[e] + e;
-}
-__global__ void k_dd_count(const DedupParams P) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= P.ns) return;
-  int e;
-  dd_count(P, t, dd_table(P, t, e));
-}
-__global__ void k_dd_fill(const DedupParams P) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= P.ns) return;
-  int e;
-  dd_fill(P, t, dd_table(P, t, e), P.owners);
-}
-__global__ void k_dd_conflicts(const DedupParams P) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= P.ns) return;
-  int e;
-  const unsigned* cnt = dd_table(P, t, e);
-  // hit 0's owners start where the previous table's extra entry points
-  const unsigned start0 = (P.hit_off[e] + e == 0) ? 0u : cnt[-1];
-  dd_conflicts(P, t, cnt, start0, P.owners);
-}
-__global__ void __launch_bounds__(DEDUP_THREADS) k_dd_rounds(const DedupParams P) {
-  const int e = blockIdx.x;
-  dd_rounds(Rounds{P.n_conf, P.conf, P.state, P.keep, P.status, ST_DEDUP_ROUNDS, P.max_rounds}, P.seed_off[e],
-            P.seed_off[e + 1]);
+__global__ void __launch_bounds__(DEDUP_THREADS) k_dd_rounds(const DedupParams P, int e_begin) {
+  const int e = e_begin + blockIdx.x;
+  dd_rounds(Rounds{P.n_conf, P.conf, P.state, P.keep, P.status, ST_DEDUP_ROUNDS, P.max_rounds},
+            P.seed_off ? P.seed_off[e] : 0, P.seed_off ? P.seed_off[e + 1] : P.ns);
 }
 
 // ------------------------------------------------------------ seed cleaning
@@ -432,27 +374,19 @@ __global__ void __launch_bounds__(DEDUP_THREADS) k_sc_resolve(const SeedCleanPar
 
 }  // namespace
 
-cudaError_t launch_dedup(const DedupParams& P, int n_events, cudaStream_t st) {
+cudaError_t launch_dedup(const DedupParams& P, int t_begin, int t_end, int e_begin, int n_events, size_t head_begin,
+                         size_t n_heads, cudaStream_t st) {
   if (n_events <= 0) return cudaSuccess;
-  k_dedup<<<n_events, DEDUP_THREADS, 0, st>>>(P);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_dedup_batched(const DedupParams& P, int n_events, int n_hits, unsigned* scan_tmp,
-                                 size_t scan_tmp_elems_, cudaStream_t st) {
-  if (n_events <= 0) return cudaSuccess;
-  const size_t n_tab = (size_t)n_hits + n_events;
-  cudaError_t e = cudaMemsetAsync(P.hit_cnt, 0, sizeof(unsigned) * (n_tab + 1), st);
-  if (e != cudaSuccess) return e;
-  const int threads = 256, blocks = (P.ns + threads - 1) / threads;
-  if (P.ns > 0) k_dd_count<<<blocks, threads, 0, st>>>(P);
-  e = scan_exclusive_inplace(P.hit_cnt, n_tab, 0u, scan_tmp, scan_tmp_elems_, st);
-  if (e != cudaSuccess) return e;
-  if (P.ns > 0) {
-    k_dd_fill<<<blocks, threads, 0, st>>>(P);
-    k_dd_conflicts<<<blocks, threads, 0, st>>>(P);
+  const int n = t_end - t_begin;
+  if (n > 0) {
+    const cudaError_t e = cudaMemsetAsync(P.head + head_begin, 0xFF, sizeof(unsigned) * n_heads, st);
+    if (e != cudaSuccess) return e;
+    const size_t entries = (size_t)n * P.L;
+    k_dd_build<<<(unsigned)((entries + DD_THREADS - 1) / DD_THREADS), DD_THREADS, 0, st>>>(P, t_begin, t_end);
+    constexpr int PER = DD_THREADS / DD_LANES;
+    k_dd_conflicts<<<(n + PER - 1) / PER, DD_THREADS, 0, st>>>(P, t_begin, t_end);
   }
-  k_dd_rounds<<<n_events, DEDUP_THREADS, 0, st>>>(P);
+  k_dd_rounds<<<n_events, DEDUP_THREADS, 0, st>>>(P, e_begin);
   return cudaGetLastError();
 }
 
@@ -485,14 +419,14 @@ cudaError_t launch_seed_clean(const SeedCleanParams& P, int pos_begin, int pos_e
 // results, so such calls must be ordered.
 namespace {
 
-constexpr size_t NA_CNT_BYTES = ((size_t)(KF_NOALLOC_MAX_HITS + 1) * 4 + 255) / 256 * 256;
-constexpr size_t NA_OWN_BYTES = (size_t)KF_NOALLOC_MAX_TRACKS * KF_MAX_LAYERS * 4;
+constexpr size_t NA_HEAD_BYTES = ((size_t)(KF_NOALLOC_MAX_HITS) * 4 + 255) / 256 * 256;
+constexpr size_t NA_NEXT_BYTES = (size_t)KF_NOALLOC_MAX_TRACKS * KF_MAX_LAYERS * 4;
 constexpr size_t NA_CONF_BYTES = (size_t)KF_NOALLOC_MAX_TRACKS * DEDUP_CONF_CAP * 4;
 constexpr size_t NA_NCONF_BYTES = (size_t)KF_NOALLOC_MAX_TRACKS * 4;
 constexpr size_t NA_STATE_BYTES = ((size_t)KF_NOALLOC_MAX_TRACKS + 255) / 256 * 256;
-constexpr size_t NA_MISC_BYTES = 256;  // event offsets and the status word
+constexpr size_t NA_MISC_BYTES = 256;  // the status word
 constexpr size_t NA_BYTES =
-    NA_CNT_BYTES + NA_OWN_BYTES + NA_CONF_BYTES + NA_NCONF_BYTES + NA_STATE_BYTES + NA_MISC_BYTES;
+    NA_HEAD_BYTES + NA_NEXT_BYTES + NA_CONF_BYTES + NA_NCONF_BYTES + NA_STATE_BYTES + NA_MISC_BYTES;
 
 static __device__ __align__(256) unsigned char kf_noalloc_scratch[NA_BYTES];
 
@@ -500,18 +434,6 @@ static __device__ __align__(256) unsigned char kf_noalloc_scratch[NA_BYTES];
 constexpr int NA_MAX_DEVICES = 64;
 std::mutex na_mutex;
 unsigned char* na_ptr[NA_MAX_DEVICES] = {};
-
-// Writes the one-event offsets and clears the status words.
-__global__ void k_noalloc_prep(int* misc, int n_tracks, int n_hits, int* user_status) {
-  if (threadIdx.x == 0) {
-    misc[0] = 0;         // seed_off
-    misc[1] = n_tracks;
-    misc[2] = 0;         // hit_off
-    misc[3] = n_hits;
-    misc[4] = ST_OK;     // status
-    if (user_status) *user_status = ST_OK;
-  }
-}
 
 }  // namespace
 
@@ -542,27 +464,24 @@ extern "C" int kf_remove_duplicates_noalloc(int n_tracks, int n_layers, int n_hi
     }
     base = na_ptr[dev];
   }
-  int* misc = reinterpret_cast<int*>(base + NA_BYTES - NA_MISC_BYTES);
   DedupParams D;
   D.out_hits = hits;
   D.out_n = n_found;
   D.out_chi2 = chi2;
-  D.seed_off = misc;
-  D.seed_event = nullptr;  // single-event launch only
-  D.hit_off = misc + 2;
+  D.seed_off = nullptr;  // one event of n_tracks tracks
+  D.seed_event = nullptr;
+  D.hit_off = nullptr;
   D.L = n_layers;
   D.ns = n_tracks;
   D.frac = dup_shared_frac;
-  D.e_begin = 0;
-  D.hit_cnt = reinterpret_cast<unsigned*>(base);
-  D.owners = reinterpret_cast<int*>(base + NA_CNT_BYTES);
-  D.conf = reinterpret_cast<int*>(base + NA_CNT_BYTES + NA_OWN_BYTES);
-  D.n_conf = reinterpret_cast<int*>(base + NA_CNT_BYTES + NA_OWN_BYTES + NA_CONF_BYTES);
-  D.state = base + NA_CNT_BYTES + NA_OWN_BYTES + NA_CONF_BYTES + NA_NCONF_BYTES;
+  D.head = reinterpret_cast<unsigned*>(base);
+  D.next = reinterpret_cast<unsigned*>(base + NA_HEAD_BYTES);
+  D.conf = reinterpret_cast<int*>(base + NA_HEAD_BYTES + NA_NEXT_BYTES);
+  D.n_conf = reinterpret_cast<int*>(base + NA_HEAD_BYTES + NA_NEXT_BYTES + NA_CONF_BYTES);
+  D.state = base + NA_HEAD_BYTES + NA_NEXT_BYTES + NA_CONF_BYTES + NA_NCONF_BYTES;
   D.keep = keep;
-  D.status = status ? status : misc + 4;
-  k_noalloc_prep<<<1, 32, 0, st>>>(misc, n_tracks, n_hits, status);
-  if (cudaGetLastError() != cudaSuccess) return KF_ERR_CUDA;
-  if (launch_dedup(D, 1, st) != cudaSuccess) return KF_ERR_CUDA;
+  D.status = status ? status : reinterpret_cast<int*>(base + NA_BYTES - NA_MISC_BYTES);
+  if (cudaMemsetAsync(D.status, 0, sizeof(int), st) != cudaSuccess) return KF_ERR_CUDA;
+  if (launch_dedup(D, 0, n_tracks, 0, 1, 0, (size_t)n_hits, st) != cudaSuccess) return KF_ERR_CUDA;
   return KF_OK;
 }

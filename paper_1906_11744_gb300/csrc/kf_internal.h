@@ -89,15 +89,14 @@ struct DedupParams {
   const int* out_hits;   // [ns][L]
   const int* out_n;
   const float* out_chi2;
-  const int* hit_off;
-  const int* seed_off;   // [n_events + 1]
-  const int* seed_event; // [ns] (batched launch)
-  int L;
+  const int* hit_off;    // [n_events + 1]
+  const int* seed_off;   // [n_events + 1]; null: one event of ns tracks
+  const int* seed_event; // [ns]; null: one event
+  int L;                 // at most 64
   int ns;
   float frac;
-  int e_begin;           // first event of this launch (one block per event)
-  unsigned* hit_cnt;     // [n_hits + n_events]
-  int* owners;           // [ns * L]
+  unsigned* head;        // event e's hit h at [hit_off[e] + e + h]: the last entry of its owner list
+  unsigned* next;        // [ns * L] the entry before
   int* conf;             // [ns * DEDUP_CONF_CAP]
   int* n_conf;           // [ns]
   unsigned char* state;  // [ns]
@@ -263,17 +262,12 @@ cudaError_t launch_find_careful_disk(const FindParams& P, int lanes, int grid, c
 cudaError_t launch_bin(const BinParams& P, size_t bin_begin, size_t n_bins, unsigned first_pos, int max_event_hits,
                        unsigned* scan_tmp, size_t scan_tmp_elems, cudaStream_t st);
 size_t scan_tmp_elems(size_t n);
-// Exclusive scan of cnt[0..n) in place plus add; cnt[n] = total + add.
-// tmp: scan_tmp_elems(n) entries.
-cudaError_t scan_exclusive_inplace(unsigned* cnt, size_t n, unsigned add, unsigned* tmp, size_t tmp_elems,
-                                   cudaStream_t st);
 size_t bin_group_elems(int n_events, int n_layers, int n_eta, int n_phi);
 // kf_dedup.cu
-cudaError_t launch_dedup(const DedupParams& P, int n_events, cudaStream_t st);
-// Whole batch: hit_cnt holds n_hits + n_events + 1 entries; scan_tmp
-// scan_tmp_elems(n_hits + n_events) entries.
-cudaError_t launch_dedup_batched(const DedupParams& P, int n_events, int n_hits, unsigned* scan_tmp,
-                                 size_t scan_tmp_elems, cudaStream_t st);
+// Tracks [t_begin, t_end), those of events [e_begin, e_begin + n_events), whose
+// list heads are head[head_begin, head_begin + n_heads).
+cudaError_t launch_dedup(const DedupParams& P, int t_begin, int t_end, int e_begin, int n_events, size_t head_begin,
+                         size_t n_heads, cudaStream_t st);
 // Seed cleaning of the seeds at positions [pos_begin, pos_end) of the theta
 // order, which are those of events [e_begin, e_begin + n_events).
 cudaError_t launch_seed_clean(const SeedCleanParams& P, int pos_begin, int pos_end, int e_begin, int n_events,
