@@ -27,6 +27,8 @@ struct kf_ctx {
   kf_config cfg;
   DevGeom g;
   int lanes = 0, threads = 0, persistent = 1, per_event = 0, regcap = 0;
+  bool auto_cap = false;  // block size and register budget left to the library
+  int cap_blocks_per_sm = 1;  // resident blocks of the register-capped kernel
   int num_sms = 0;
   int blocks_per_sm = 1;
   int n_events = 0, n_hits = 0, n_seeds = 0, n_seed_events = -1, max_event_hits = 0;
@@ -38,7 +40,8 @@ struct kf_ctx {
   DevBuf hb, bin_cnt, bin_key, bin_rank, scan_tmp, bin_grouped, bin_gtab;
   // finding
   DevBuf out_hits, out_n, out_chi2, out_p, out_C, keep, queue, counters, status, tangent, seed_order, check;
-  DevBuf sfit, sflag, skeys, x0map;
+  DevBuf sfit, sflag, skeys, x0map, rec;
+  int rec_cap = 0;
   // duplicate removal scratch (the conflict lists also serve seed cleaning)
   DevBuf dd_head, dd_next, dd_conf, dd_nconf, dd_state;
   // seed cleaning
@@ -265,6 +268,7 @@ int kf_create(const kf_detector* det, const kf_config* cfg, kf_ctx** out) {
   ctx->persistent = cfg->persistent ? 1 : 0;
   ctx->per_event = cfg->per_event ? 1 : 0;
   ctx->regcap = cfg->find_regcap;
+  ctx->auto_cap = cfg->block_threads == 0 && cfg->find_regcap == 0;
   DevGeom& g = ctx->g;
   std::memset(&g, 0, sizeof(g));
   g.n_layers = det->n_layers;
@@ -307,6 +311,8 @@ int kf_create(const kf_detector* det, const kf_config* cfg, kf_ctx** out) {
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess)
     e = find_prepare(ctx->lanes, ctx->regcap, ctx->threads, ctx->g, &ctx->blocks_per_sm);
+  if (e == cudaSuccess && ctx->auto_cap)
+    e = find_prepare(ctx->lanes, 1, ctx->threads, ctx->g, &ctx->cap_blocks_per_sm);
   if (e == cudaSuccess) e = grow(ctx->align4, sizeof(Align4) * KF_MAX_LAYERS);
   if (e == cudaSuccess) {
     // z edges of the eta bins per layer: edge_k = R sinh(-eta_max + k * 2 eta_max / n_eta)
@@ -371,7 +377,7 @@ static std::vector<DevBuf*> all_bufs(kf_ctx* ctx) {
                     &ctx->careful_count, &ctx->adj_align_acc, &ctx->adj_align, &ctx->adj_hits,
                     &ctx->adj_seed, &ctx->careful_flag, &ctx->ckpt, &ctx->sc_kin, &ctx->sc_seed,
                     &ctx->clean_order, &ctx->kept_cnt, &ctx->sc_list, &ctx->sc_list_cnt, &ctx->sfit,
-                    &ctx->sflag, &ctx->skeys, &ctx->x0map, &ctx->fit_order, &ctx->dbl_list};
+                    &ctx->sflag, &ctx->skeys, &ctx->x0map, &ctx->rec, &ctx->fit_order, &ctx->dbl_list};
 }
 
 int kf_destroy(kf_ctx* ctx) {
@@ -477,6 +483,10 @@ int kf_load_seeds(kf_ctx* ctx, int n_events, const int* ev_offsets, const float*
   CK(grow(ctx->seed_order, sizeof(int) * (size_t)n));
   CK(grow(ctx->sfit, sizeof(float) * 29 * (size_t)n));
   CK(grow(ctx->sflag, (size_t)n));
+  // records of given-up seeds: about 0.3% of them; room for a thirty-second
+  const int rec_cap = n / 32 + 64;
+  CK(grow(ctx->rec, sizeof(unsigned) * find_record_words(ctx->g.n_plan, ctx->g.max_cands) * (size_t)rec_cap));
+  ctx->rec_cap = rec_cap;
   CK(grow(ctx->skeys, sizeof(unsigned long long) * ctx->g.max_cands * (size_t)n));
   CK(grow(ctx->out_chi2, sizeof(float) * (size_t)n));
   CK(grow(ctx->out_p, sizeof(float) * 6 * (size_t)n));
@@ -631,6 +641,8 @@ static FindParams find_params(kf_ctx* ctx) {
   P.out_C = ptr<float>(ctx->out_C);
   P.queue = ptr<unsigned>(ctx->queue);
   P.tangent_list = ptr<int>(ctx->tangent);
+  P.rec = ptr<unsigned>(ctx->rec);
+  P.rec_cap = ctx->rec_cap;
   P.sfit = ptr<float>(ctx->sfit);
   P.sflag = ptr<unsigned char>(ctx->sflag);
   P.skeys = ptr<unsigned long long>(ctx->skeys);
@@ -706,6 +718,13 @@ static int careful_grid(const kf_ctx* ctx, int n_seeds) {
   return std::max(1, std::min(2 * ctx->num_sms, (n_seeds / 50 + 11) / 12));
 }
 
+// With block size and register budget left to the library, a launch of more
+// candidate places than this takes the register-capped finding kernel (five
+// blocks per SM, no records of given-up seeds): its main pass is 7% faster on
+// a full chip, which from about 0.75 ms of finding on outweighs the 60 us that
+// the records save the careful pass.
+constexpr long long AUTO_CAP_CANDS = 600000;
+
 int kf_find_tracks(kf_ctx* ctx, void* stream) {
   if (!ctx) return KF_ERR_ARG;
   if (ctx->n_hits < 0 || ctx->n_seed_events != ctx->n_events || ctx->n_events < 1)
@@ -714,7 +733,11 @@ int kf_find_tracks(kf_ctx* ctx, void* stream) {
   const size_t cells = (size_t)ctx->g.n_surf * ctx->g.n_eta * ctx->g.n_phi;
   CK(cudaMemsetAsync(ctx->counters.p, 0, 8 * KF_N_COUNTERS, st));
   CK(cudaMemsetAsync(ctx->keep.p, 1, (size_t)ctx->n_seeds, st));
-  const int grid_cap = ctx->num_sms * ctx->blocks_per_sm;
+  auto find_main = [&](const FindParams& P) {
+    const bool cap = ctx->regcap || (ctx->auto_cap && (long long)(P.s_end - P.s_begin) * ctx->g.max_cands > AUTO_CAP_CANDS);
+    const int bps = cap && !ctx->regcap ? ctx->cap_blocks_per_sm : ctx->blocks_per_sm;
+    return launch_find_main(P, ctx->lanes, cap, ctx->threads, ctx->num_sms * bps, st);
+  };
   if (!ctx->per_event) {
     BinParams B = bin_params(ctx);
     stage_mark(ctx, 0, st);
@@ -731,7 +754,7 @@ int kf_find_tracks(kf_ctx* ctx, void* stream) {
     }
     CK(cudaMemsetAsync(ctx->queue.p, 0, 64, st));
     stage_mark(ctx, 2, st);
-    CK(launch_find_main(P, ctx->lanes, ctx->regcap, ctx->threads, grid_cap, st));
+    CK(find_main(P));
     CK(launch_find_careful(P, ctx->lanes, careful_grid(ctx, P.s_end - P.s_begin), st));
     stage_mark(ctx, 3, st);
   } else {
@@ -751,7 +774,7 @@ int kf_find_tracks(kf_ctx* ctx, void* stream) {
         P.kept_cnt = ptr<int>(ctx->kept_cnt);
       }
       CK(cudaMemsetAsync(ctx->queue.p, 0, 64, st));
-      CK(launch_find_main(P, ctx->lanes, ctx->regcap, ctx->threads, grid_cap, st));
+      CK(find_main(P));
       CK(launch_find_careful(P, ctx->lanes, careful_grid(ctx, P.s_end - P.s_begin), st));
     }
   }
@@ -1168,6 +1191,7 @@ int kf_autotune(kf_ctx* ctx, float* results, int max_results, int* n_results, vo
   float best = 1e30f;
   int best_l = saved_lanes, best_t = saved_threads, best_p = saved_pers, best_b = saved_bps,
       best_rc = saved_rc;
+  ctx->auto_cap = false;  // the shape is the tuner's from here on
   int nr = 0;
   cudaEvent_t a, b;
   CK(cudaEventCreate(&a));

@@ -62,6 +62,8 @@ size_t find_smem_bytes(int threads, int n_layers, int n_eta) {
   return smem_edges(n_layers, n_eta) + (size_t)(threads / 32) * smem_per_warp(KF_MAX_CANDS, false, n_layers);
 }
 
+size_t find_record_words(int n_plan, int max_cands) { return (size_t)(REC_HIST + n_plan) * max_cands; }
+
 bool find_lanes_supported(int lanes) {
   return lanes == 4 || lanes == 6 || lanes == 8 || lanes == 10 || lanes == 12 || lanes == 16;
 }

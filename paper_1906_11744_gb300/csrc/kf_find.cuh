@@ -85,11 +85,11 @@ constexpr float WIN_Z_ABS = 1e-4f;    // cm
 // and radial direction) are propagated in double: the FP32 error of the
 // transported covariance grows as 1/cos^4 and near the turning radius of a
 // looper it can leave the prediction without a positive definite S.  The
-// main pass gives up a seed whose candidates meet such a crossing (after that
-// layer its lanes go idle) and lists it; a careful pass after it (the same
-// kernel with CAREFUL) redoes the listed seeds with those propagations in
-// double, so that the double code and its registers stay out of the main
-// pass.  The threshold for the finding is 0.2: on the PU-200 batch every
+// main pass gives up a seed whose candidates meet such a crossing (before that
+// layer's search; its lanes go idle), lists it and leaves a record of its
+// candidates; a careful pass after it (the same kernel with CAREFUL) takes the
+// listed seeds on from there with those propagations in double, so that the
+// double code and its registers stay out of the main pass.  The threshold for the finding is 0.2: on the PU-200 batch every
 // threshold from 0.1 to 0.5 gives the oracle's hit lists for the most tangent
 // loopers, and no prediction without a positive definite S, while the double
 // work (FP64 runs at a small fraction of the FP32 rate) grows tenfold from 0.2
@@ -267,6 +267,16 @@ __device__ __forceinline__ Window window_disk(const FindParams& P, const float (
   w.b1 = min(b0 + span, nphi);
   w.b2 = b0 + span - nphi;
   return w;
+}
+
+// What the main pass leaves of a seed it gives up in the middle of its search,
+// at the seed's place in the list: per candidate the words below (state, chi2
+// sum, counts and flags, the task's counters), then the history's columns so
+// far.  Places at rec_cap or beyond have none (searched again from the seed).
+constexpr unsigned GIVEN_UP_RECORD = 0x80000000u;  // flag of a list entry
+constexpr int REC_CHI2 = 27, REC_META = 28, REC_IT = 29, REC_COUNT = 30, REC_HIST = 38;
+__device__ __forceinline__ unsigned* given_up_record(const FindParams& P, int j, int HL) {
+  return P.rec + (size_t)j * (REC_HIST + HL) * P.g.max_cands;
 }
 
 // Tests every hit of the window (cell offsets off of the event and layer)
@@ -584,12 +594,26 @@ __global__ void __launch_bounds__(SEED_THREADS) k_seed_fit(const FindParams P) {
   }
 }
 
+// Which main kernels leave records: those at the compiler's register count,
+// which the launches that do not fill the chip run.  There the careful pass is
+// a good part of the time, and taking a seed on from the surface instead of
+// from its seed saves 60 us (8,000-seed event: 0.28 -> 0.22 ms of finding).
+// In the register-capped kernels, for large batches, the record's code costs
+// more than it saves (100 events x 8,000 seeds: 7.42 -> 7.73 ms).  The disk
+// kernels keep none: their main and careful code round some FP32 steps
+// differently, and a near-tangent covariance amplifies that.
+__host__ __device__ constexpr bool keeps_records(int cap, bool disk) { return cap == 0 && !disk; }
+
 // EL: the detector has energy loss (the main pass without it carries none of
 // its code; the careful pass always does).  DISK: the detector has endcap
 // disks (region plans, disk surfaces).
 template <int G, int CAP, bool CAREFUL, bool EL, bool DISK = false>
-__global__ void __launch_bounds__(CAP ? 128 : 256, CAP ? 5 : 1) k_find(const FindParams P) {
+__global__ void __launch_bounds__(CAP ? 128 : 256, CAP ? 5 : CAREFUL ? 1 : 2) k_find(const FindParams P) {
   constexpr int W = 32 / G;  // seeds per warp
+  // The main pass leaves a record of a seed it gives up (REC) and the careful
+  // pass takes it on (RESUME): see keeps_records.
+  constexpr bool REC = !CAREFUL && keeps_records(CAP, DISK);
+  constexpr bool RESUME = CAREFUL && !DISK;
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -621,8 +645,13 @@ __global__ void __launch_bounds__(CAP ? 128 : 256, CAP ? 5 : 1) k_find(const Fin
   int* hist = reinterpret_cast<int*>(ws + SL + SG + SMEM_SLOT);
   const int N = g.max_cands;
   const int n_seed_range = CAREFUL ? (int)P.queue[2] : P.s_end - P.s_begin;
-  const int n_tasks = (n_seed_range + W - 1) / W;
   const int warps_per_block = blockDim.x >> 5;
+  // seeds per warp: the careful pass spreads a short list over its warps (a
+  // double-precision instruction takes its unit 64 clocks whatever the number
+  // of active lanes, and the seeds of a warp reach them at different layers)
+  const int WT =
+      CAREFUL ? min(W, (n_seed_range + (int)gridDim.x * warps_per_block - 1) / ((int)gridDim.x * warps_per_block)) : W;
+  const int n_tasks = n_seed_range > 0 ? (n_seed_range + WT - 1) / WT : 0;
   unsigned* const queue = P.queue + (CAREFUL ? 1 : 0);
   // Counters: per-warp sums in shared memory (lane 0 of the warp owns its
   // row), added to the global counters once when the warp ends.
@@ -646,10 +675,14 @@ __global__ void __launch_bounds__(CAP ? 128 : 256, CAP ? 5 : 1) k_find(const Fin
   while (task < n_tasks) {
     int seed;
     bool has_seed;
+    int list_pos = 0;     // careful pass: the seed's place in the list
+    bool resume = false;  // careful pass: the main pass left a record of the search
     if constexpr (CAREFUL) {
-      const int j = task * W + grp;
-      has_seed = lane_used && j < n_seed_range;
-      seed = has_seed ? P.tangent_list[j] : 0;
+      list_pos = task * WT + grp;
+      has_seed = lane_used && grp < WT && list_pos < n_seed_range;
+      const unsigned v = has_seed ? (unsigned)P.tangent_list[list_pos] : 0u;
+      seed = (int)(v & ~GIVEN_UP_RECORD);
+      resume = RESUME && (v & GIVEN_UP_RECORD) != 0u;
     } else {
       const int j = P.s_begin + task * W + grp;
       has_seed = lane_used && (j < P.s_end);
@@ -663,6 +696,10 @@ __global__ void __launch_bounds__(CAP ? 128 : 256, CAP ? 5 : 1) k_find(const Fin
     unsigned c_steps = 0, c_updates = 0, c_chi2 = 0, c_seeds = 0, c_holes = 0, c_careful = 0, c_npd = 0;
     unsigned c_dsteps = 0, c_dupdates = 0, c_dholes = 0;  // DISK: the steps, updates and holes on disks
     bool near = false, given_up = false;
+    // given up: the candidate is propagated to the surface of this iteration (0:
+    // given up by the seed kernel), was searched on it
+    bool there = false, searched = false;
+    int it_up = 0;
     // main pass: the first layer's children, found by the seed kernel (this
     // lane's child and whether their parent was carried or propagated)
     unsigned long long first_key = KEY_EMPTY;
@@ -723,12 +760,50 @@ __global__ void __launch_bounds__(CAP ? 128 : 256, CAP ? 5 : 1) k_find(const Fin
     // iterations: the three seed hits (careful pass only; the main pass starts
     // from the fitted seed), then the positions of the plan
     int n_iter = has_seed && !given_up ? 3 + (L - start) + (fwd ? g.n_disks : 0) : 0;
-    int it_end = __reduce_max_sync(0xffffffffu, n_iter);
+    int it0 = 0;             // careful pass: the group's first iteration
+    // and whether its candidate comes propagated to that surface, counted there
+    bool prop_done = false, counted = false;
+    if constexpr (RESUME) {
+      if (resume) {  // take the search on from the surface where the main pass gave it up
+        const unsigned* rec = given_up_record(P, list_pos, HL);
+        it0 = (int)rec[REC_IT * N];
+        occ = false;
+        if (gl < N) {
+#pragma unroll
+          for (int k = 0; k < 6; ++k) p[k] = __uint_as_float(rec[k * N + gl]);
+#pragma unroll
+          for (int k = 0; k < 21; ++k) C[k] = __uint_as_float(rec[(6 + k) * N + gl]);
+          chi2 = __uint_as_float(rec[REC_CHI2 * N + gl]);
+          const unsigned m = rec[REC_META * N + gl];
+          nfound = (int)(m & 255u);
+          nholes = (int)((m >> 8) & 255u);
+          occ = (m >> 16) & 1u;
+          finished = (m >> 17) & 1u;
+          bdone = (m >> 18) & 1u;
+          prop_done = (m >> 19) & 1u;
+          counted = (m >> 20) & 1u;
+          c_steps = rec[(REC_COUNT + 0) * N + gl];
+          c_updates = rec[(REC_COUNT + 1) * N + gl];
+          c_chi2 = rec[(REC_COUNT + 2) * N + gl];
+          c_holes = rec[(REC_COUNT + 3) * N + gl];
+          c_npd = rec[(REC_COUNT + 4) * N + gl];
+          c_dsteps = rec[(REC_COUNT + 5) * N + gl];
+          c_dupdates = rec[(REC_COUNT + 6) * N + gl];
+          c_dholes = rec[(REC_COUNT + 7) * N + gl];
+          for (int q = start; q < start + it0 - 3; ++q)
+            hist[(grp * HL + q) * G + gl] = (int)rec[(REC_HIST + q) * N + gl];
+        }
+      }
+    }
+    // the warp's iteration `itw` is iteration itw + it0 of its group, so that
+    // the near-tangent surfaces of a warp's seeds fall together
+    int it_end = __reduce_max_sync(0xffffffffu, n_iter - it0);
 
 #pragma unroll 1
-    for (int it = CAREFUL ? 0 : 3; it < it_end; ++it) {
+    for (int itw = CAREFUL ? 0 : 3; itw < it_end; ++itw) {
+      const int it = itw + it0;
       const bool in_seed = CAREFUL && it < 3;
-      const bool active = it < n_iter;
+      bool active = it < n_iter;
       const int pos = start + (it - 3);  // position in the plan (the history's column)
       const int l = in_seed ? (it == 0 ? sl0 : (it == 1 ? sl1 : sl2)) : (DISK ? plan_surface(g, pos, neg) : pos);
       const bool disk = DISK && !in_seed && is_disk(g, l);
@@ -774,7 +849,9 @@ __global__ void __launch_bounds__(CAP ? 128 : 256, CAP ? 5 : 1) k_find(const Fin
           }
           const float R = disk ? 0.f : g.radius[l];
           int pr = 1;
-          if (disk) {
+          if (RESUME && prop_done) {
+            prop_done = false;  // propagated by the main pass
+          } else if (disk) {
             // the plane step; a crossing outside the disk's radii is none
             float q[6], J[6][6];
             pr = prop_plane_jacobian<float>(p, plane_z(g, l), field_kb<float>(g, p), q, J) ? 1 : 0;
@@ -809,7 +886,15 @@ __global__ void __launch_bounds__(CAP ? 128 : 256, CAP ? 5 : 1) k_find(const Fin
               }
               c_careful++;
             } else if (pr == 1) {
-              if (!CAREFUL && cosa < FIND_CAREFUL_COS) near = true;
+              if (!CAREFUL && cosa < FIND_CAREFUL_COS) {
+                near = true;
+                if constexpr (REC) {
+#pragma unroll
+                  for (int k = 0; k < 6; ++k) bak[k] = p[k];
+#pragma unroll
+                  for (int k = 0; k < 21; ++k) bak[6 + k] = C[k];
+                }
+              }
               transport<float>(J, C);
 #pragma unroll
               for (int k = 0; k < 6; ++k) p[k] = q[k];
@@ -821,29 +906,33 @@ __global__ void __launch_bounds__(CAP ? 128 : 256, CAP ? 5 : 1) k_find(const Fin
             cls = fwd && !in_seed ? 3 : 1;
             finished = cls == 1;
             tail = make_key(nfound, chi2, gl, 1, 0);
-          } else {
+          } else if (CAREFUL || !near) {
             cls = 2;
             if (!in_seed && disk) {
-              c_steps++;
-              c_dsteps++;
+              if (!RESUME || !counted) {
+                c_steps++;
+                c_dsteps++;
+              }
               DiskFrameT<float> d;
               make_frame_disk<float>(p, C, g.vr, g.vrr, d);
               const bool spd = d.f.s00 > 0.f && d.f.si00 > 0.f && d.f.si11 > 0.f;
-              if (!spd) c_npd++;
+              if (!spd && !(RESUME && counted)) c_npd++;
               const Window w = window_disk(P, p, d.f, spd);
               const unsigned* off = P.bin_off + ((size_t)ev * S + l) * ((size_t)g.n_eta * g.n_phi);
+              const unsigned c_before = c_chi2;
               scan_window<CAREFUL, true>(P, off, w, Align4{1.f, 0.f, 0.f, 0.f}, p, d.f, nfound + 1, chi2, gl, lst,
                                          cnt, c_chi2);
+              if (RESUME && counted) c_chi2 = c_before;
               after_scan();
             } else if (!in_seed) {
-              c_steps++;
+              if (!RESUME || !counted) c_steps++;
               Frame f;
               if (CAREFUL && dbl) f = careful_frame(dst_warp + lane * 27, g.vr, g.vz);
               else make_frame<float>(p, C, g.vr, g.vz, f);
               // A prediction without a positive definite S searches no hits
               // (the careful propagation should leave none; counted).
               const bool spd = f.s00 > 0.f && f.si00 > 0.f && f.si11 > 0.f;
-              if (!spd) c_npd++;
+              if (!spd && !(RESUME && counted)) c_npd++;
               const Align4 al = P.align[l];
               const Window w = window_of(P, l, R, p, f, spd, al, s_edges);
               const unsigned* off = P.bin_off + ((size_t)ev * S + l) * ((size_t)g.n_eta * g.n_phi);
@@ -854,11 +943,38 @@ __global__ void __launch_bounds__(CAP ? 128 : 256, CAP ? 5 : 1) k_find(const Fin
                 bal = al;
                 boff = off;
               } else {
+                const unsigned c_before = c_chi2;
                 scan_window<CAREFUL>(P, off, w, al, p, f, nfound + 1, chi2, gl, lst, cnt, c_chi2);
+                if (RESUME && counted) c_chi2 = c_before;
                 after_scan();
               }
             }
           }
+        }
+      }
+      if constexpr (!CAREFUL) {
+        // A group with a near-tangent crossing gives its seed up here and its
+        // lanes go idle; with REC each candidate as it is before this surface
+        // or (there) on it, where it was propagated already.
+        const unsigned nb = __ballot_sync(0xffffffffu, near);
+        if (lane_used && ((nb >> base) & ((1u << G) - 1u))) {
+          if constexpr (REC) {
+            there = searched = cls == 2;
+            // near-tangent, or it may stop on this surface: the state before it
+            if (near || (there && nholes >= g.max_holes)) {
+              there = false;
+#pragma unroll
+              for (int k = 0; k < 6; ++k) p[k] = bak[k];
+#pragma unroll
+              for (int k = 0; k < 21; ++k) C[k] = bak[6 + k];
+            }
+            it_up = it;
+          }
+          given_up = true;
+          n_iter = 0;
+          near = active = false;
+          cls = cnt = 0;
+          tail = KEY_EMPTY;
         }
       }
       if constexpr (CAREFUL) {  // the large windows, one after another, by the whole warp
@@ -866,7 +982,9 @@ __global__ void __launch_bounds__(CAP ? 128 : 256, CAP ? 5 : 1) k_find(const Fin
         while (pend) {
           const int src = __ffs(pend) - 1;
           pend &= pend - 1;
-          const int n = coop_scan(P, src, bw, boff, bal, p, bf, nfound + 1, chi2, gl, coop_warp, lst, &c_chi2);
+          unsigned n_eval = 0;
+          const int n = coop_scan(P, src, bw, boff, bal, p, bf, nfound + 1, chi2, gl, coop_warp, lst, &n_eval);
+          if (!__shfl_sync(0xffffffffu, (int)counted, src)) c_chi2 += n_eval;
           if (lane == src) cnt = n;
         }
         if (big) after_scan();
@@ -888,15 +1006,6 @@ __global__ void __launch_bounds__(CAP ? 128 : 256, CAP ? 5 : 1) k_find(const Fin
           hit_z = __ldg(P.hz + hi);
         }
       };
-      if constexpr (!CAREFUL) {
-        // A group with a near-tangent crossing gives its seed up after this
-        // layer (its lanes go idle) and lists it for the careful pass.
-        const unsigned nb = __ballot_sync(0xffffffffu, near);
-        if (lane_used && ((nb >> base) & ((1u << G) - 1u)) && !given_up) {
-          given_up = true;
-          n_iter = min(n_iter, it + 1);
-        }
-      }
       if (pre) {
         // the children of the seed's candidate, in rank order, one per lane;
         // every lane holds their parent's state already
@@ -1088,12 +1197,11 @@ __global__ void __launch_bounds__(CAP ? 128 : 256, CAP ? 5 : 1) k_find(const Fin
       // empty would only carry them on, each to its own slot, layer after
       // layer: its seed's search ends here (the backtrack starts from the
       // last layer searched), and the warp ends with its last live group.
-      if (!in_seed) {
-        const unsigned live = __ballot_sync(0xffffffffu, active && occ && !finished);
-        if (lane_used && active && !((live >> base) & ((1u << G) - 1u))) n_iter = min(n_iter, it + 1);
-        it_end = __reduce_max_sync(0xffffffffu, n_iter);
-      }
-      if constexpr (DISK) {
+      if constexpr (RESUME) counted = false;
+      const unsigned live = __ballot_sync(0xffffffffu, active && occ && !finished);
+      if (!in_seed && lane_used && active && !((live >> base) & ((1u << G) - 1u))) n_iter = min(n_iter, it + 1);
+      it_end = __reduce_max_sync(0xffffffffu, n_iter - it0);
+      if constexpr (DISK && !CAREFUL) {
         // A forward candidate that passed a barrel layer passes every later
         // one: it moves outward from its last crossing, so a larger radius
         // comes later along the helix (or never), and |z|, already beyond
@@ -1101,13 +1209,13 @@ __global__ void __launch_bounds__(CAP ? 128 : 256, CAP ? 5 : 1) k_find(const Fin
         // passed one, the warp goes on at the first disk of its plans; each
         // position skipped carries every candidate in its slot (what the
         // passes would do).
-        if (!in_seed && __any_sync(0xffffffffu, lane_used && active && occ && !finished) &&
+        if (__any_sync(0xffffffffu, lane_used && active && occ && !finished) &&
             !__any_sync(0xffffffffu, lane_used && active && occ && !finished && !bdone)) {
           const int first_disk = __reduce_min_sync(0xffffffffu, lane_used && active ? 3 + (L - start) : 0x7fffffff);
           if (first_disk > it + 1 && first_disk != 0x7fffffff) {
             for (int q = it + 1; q < first_disk; ++q)
               if (lane_used && q < n_iter) hist[(grp * HL + start + (q - 3)) * G + gl] = gl << 24;
-            it = first_disk - 1;
+            itw = first_disk - 1;
           }
         }
       }
@@ -1122,13 +1230,43 @@ __global__ void __launch_bounds__(CAP ? 128 : 256, CAP ? 5 : 1) k_find(const Fin
         c_npd += c >> 31;
       }
     }
-    if (given_up) {
-      if (has_seed && gl == 0) {
-        P.tangent_list[atomicAdd(P.queue + 2, 1u)] = seed;
-        ++c_redo;
+    if constexpr (!CAREFUL) {
+      if (__any_sync(0xffffffffu, given_up)) {  // list the seeds given up, with a record of their searches
+        unsigned j = 0;
+        if (given_up && gl == 0) {
+          j = atomicAdd(P.queue + 2, 1u);
+          P.tangent_list[j] =
+              (int)((unsigned)seed | (REC && it_up > 0 && j < (unsigned)P.rec_cap ? GIVEN_UP_RECORD : 0u));
+          ++c_redo;
+        }
+        if constexpr (REC) j = __shfl_sync(0xffffffffu, j, base);
+        if (given_up) {
+          if (REC && it_up > 0 && gl < N && j < (unsigned)P.rec_cap) {
+            unsigned* rec = given_up_record(P, (int)j, HL) + gl;
+#pragma unroll
+            for (int k = 0; k < 6; ++k) rec[k * N] = __float_as_uint(p[k]);
+#pragma unroll
+            for (int k = 0; k < 21; ++k) rec[(6 + k) * N] = __float_as_uint(C[k]);
+            rec[REC_CHI2 * N] = __float_as_uint(chi2);
+            rec[REC_META * N] = (unsigned)nfound | ((unsigned)nholes << 8) | (occ ? 1u << 16 : 0u) |
+                                (finished ? 1u << 17 : 0u) | (bdone ? 1u << 18 : 0u) | (there ? 1u << 19 : 0u) |
+                                (searched ? 1u << 20 : 0u);
+            rec[REC_IT * N] = (unsigned)it_up;
+            rec[(REC_COUNT + 0) * N] = c_steps;
+            rec[(REC_COUNT + 1) * N] = c_updates;
+            rec[(REC_COUNT + 2) * N] = c_chi2;
+            rec[(REC_COUNT + 3) * N] = c_holes;
+            rec[(REC_COUNT + 4) * N] = c_npd;
+            rec[(REC_COUNT + 5) * N] = c_dsteps;
+            rec[(REC_COUNT + 6) * N] = c_dupdates;
+            rec[(REC_COUNT + 7) * N] = c_dholes;
+            for (int q = start; q < start + it_up - 3; ++q)
+              rec[(REC_HIST + q) * N] = (unsigned)hist[(grp * HL + q) * G + gl];
+          }
+          c_steps = c_updates = c_chi2 = c_seeds = c_holes = c_npd = 0;
+          c_dsteps = c_dupdates = c_dholes = 0;
+        }
       }
-      c_steps = c_updates = c_chi2 = c_seeds = c_holes = c_npd = 0;
-      c_dsteps = c_dupdates = c_dholes = 0;
     }
     // Counters of the task: summed over the warp into its shared row.
 #pragma unroll
@@ -1208,20 +1346,31 @@ __host__ auto main_kernel() {
   else return k_find<G, CAP, false, EL, false>;
 }
 
+// Lets kernel fn take `need` bytes of dynamic shared memory.  The limit is the
+// kernel's, shared by every context, so it is set to the device's and not to
+// one context's need.
+inline cudaError_t allow_smem(const void* fn, size_t need) {
+  int dev = 0, most = 0;
+  cudaFuncAttributes fa;
+  cudaError_t err = cudaGetDevice(&dev);
+  if (err == cudaSuccess) err = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (err == cudaSuccess) err = cudaFuncGetAttributes(&fa, fn);
+  if (err != cudaSuccess) return err;
+  const size_t limit = (size_t)most - fa.sharedSizeBytes;
+  if (need > limit) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit);
+}
+
 // n_layers: barrel layers (the eta-edge table); n_hist: history columns (the
 // longest plan).
 template <int G, int CAP, bool DISK>
 cudaError_t prepare_t(int threads, int n_layers, int n_hist, int n_eta, int* blocks_per_sm) {
   const size_t smem = smem_edges(n_layers, n_eta) + (size_t)(threads / 32) * smem_per_warp(G, false, n_hist);
-  cudaError_t err =
-      cudaFuncSetAttribute(main_kernel<G, CAP, DISK, false>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (err == cudaSuccess && !DISK)
-    err = cudaFuncSetAttribute(main_kernel<G, CAP, DISK, true>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem);
+  cudaError_t err = allow_smem((const void*)main_kernel<G, CAP, DISK, false>(), smem);
+  if (err == cudaSuccess && !DISK) err = allow_smem((const void*)main_kernel<G, CAP, DISK, true>(), smem);
   if (err == cudaSuccess)
-    err = cudaFuncSetAttribute(k_find<G, 0, true, true, DISK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)(smem_edges(n_layers, n_eta) +
-                                     (CAREFUL_THREADS / 32) * smem_per_warp_k(G, n_hist, true)));
+    err = allow_smem((const void*)k_find<G, 0, true, true, DISK>,
+                     smem_edges(n_layers, n_eta) + (CAREFUL_THREADS / 32) * smem_per_warp_k(G, n_hist, true));
   if (err != cudaSuccess) return err;
   cudaFuncAttributes fa;
   err = cudaFuncGetAttributes(&fa, main_kernel<G, CAP, DISK, false>());

@@ -56,6 +56,8 @@ struct FindParams {
   unsigned* queue;           // [3] work counters of the main and careful passes and the
                              // number of listed seeds (zeroed before the launch)
   int* tangent_list;         // [ns] seeds the main pass left to the careful pass
+  unsigned* rec;             // [rec_cap][find_record_words()] what it left of their searches
+  int rec_cap;
   float* sfit;               // [29][ns] seed kernel: the state the first layer's children come
                              // from (p, C), the seed's chi2 sum, the first layer's counts
   unsigned long long* skeys; // [max_cands][ns] seed kernel: the first layer's children (keys)
@@ -249,6 +251,7 @@ cudaError_t launch_find_careful(const FindParams& P, int lanes, int grid, cudaSt
 cudaError_t launch_seed_order(const float* theta, const int* seed_off, int n_events, int* order, cudaStream_t st);
 size_t find_smem_bytes(int threads, int n_layers, int n_eta);
 bool find_lanes_supported(int lanes);
+size_t find_record_words(int n_plan, int max_cands);  // words of a seed's record (FindParams::rec)
 // Sets the dynamic shared-memory limit of the kernel variant (must run
 // outside stream capture) and reports resident blocks per SM.
 cudaError_t find_prepare(int lanes, int regcap, int threads, const DevGeom& g, int* blocks_per_sm);

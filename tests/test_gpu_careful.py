@@ -9,7 +9,7 @@ import numpy as np
 import pytest
 
 import oracle
-from kfhelp import cov_close, param_close, tracker_for
+from kfhelp import audit_mismatch, cov_close, found_cov_close, param_close, tracker_for
 from synth import make_batch
 from synth.events import true_hit_lists
 
@@ -43,5 +43,46 @@ def test_careful_fit_list_sizes(n, loose):
     ok = (st == 0) & (fit["status"] == 0)
     okp, ep = param_close(fit["params"].T[ok], p[ok])
     okc, ec = cov_close(fit["cov"].T[ok], C[ok], p[ok])
+    assert okp.all(), ep
+    assert okc.all(), ec
+
+
+@pytest.mark.parametrize("cap", [0, 1])
+@pytest.mark.parametrize("n,loose,holes,cands", [(1, True, 3, 6), (40, True, 3, 4), (900, True, 3, 10),
+                                                 (9000, False, 3, 6), (9000, False, 0, 10), (9000, False, 1, 16)])
+def test_careful_finding(n, loose, holes, cands, cap):
+    """Seeds given up by the main pass, with (cap 0) and without a record of
+    their search: lists of a few seeds and of more than there are warps, and
+    candidates without holes left, which stop on the surface with the state
+    before it.  Hit lists and work counters equal the oracle's where the two
+    agree on every seed looked at: those that meet a near-tangent crossing."""
+    b = make_batch("c1", tracks=n)
+    if loose:
+        for i in range(6):
+            b.cov[i * 6 - i * (i - 1) // 2] = LOOSE_VAR[i]
+    t = tracker_for(b, max_cands=cands, max_holes=holes, find_regcap=cap)
+    t.find_tracks()
+    g = t.counters()
+    trk = t.get_tracks()
+    t.close()
+    assert g["redone"] == b.n_seeds if loose else 1 <= g["redone"] < b.n_seeds
+    # the low-pT tail: every seed that can meet a tangent crossing inside the barrel
+    sel = np.arange(b.n_seeds) if loose else np.argsort(-np.abs(b.params[3]))[:max(100, b.n_seeds // 25)]
+    from concurrent.futures import ThreadPoolExecutor
+    with ThreadPoolExecutor(8) as ex:
+        ref = list(ex.map(lambda s: oracle.find_event(b, 0, max_cands=cands, max_holes=holes, seeds=(int(s), int(s) + 1)),
+                          sel))
+    same = np.array([np.array_equal(trk["hits"][s], r["hits"][0]) for s, r in zip(sel, ref)])
+    for s, r in zip(sel[~same], [r for r, k in zip(ref, same) if not k]):
+        ok, kind, rel = audit_mismatch(b, 0, int(s), trk["hits"][s], r["hits"][0])
+        assert ok, (int(s), kind, rel)
+    assert same.mean() >= 0.98
+    if loose and same.all():
+        for k in ("steps", "updates", "holes"):
+            assert abs(g[k] - sum(r["counters"][k] for r in ref)) <= 1e-3 * g[k]
+    p = np.concatenate([r["p"] for r in ref])[same]
+    C = np.concatenate([r["C"] for r in ref])[same]
+    okp, ep = param_close(trk["params"].T[sel][same], p)
+    okc, ec = found_cov_close(trk["cov"].T[sel][same], C, p)
     assert okp.all(), ep
     assert okc.all(), ec
