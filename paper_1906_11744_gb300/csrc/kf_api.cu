@@ -814,12 +814,13 @@ int kf_remove_duplicates(kf_ctx* ctx, void* stream) {
   }
   if (!ctx->per_event) {
     stage_mark(ctx, 4, st);
-    CK(launch_dedup(D, 0, ctx->n_seeds, 0, ctx->n_events, 0, (size_t)ctx->n_hits + ctx->n_events, st));
+    CK(launch_dedup(D, 0, ctx->n_seeds, 0, ctx->n_events, 0, (size_t)ctx->n_hits + ctx->n_events, false,
+                    st));
     stage_mark(ctx, 5, st);
   } else {
     for (int e = 0; e < ctx->n_events; ++e)
       CK(launch_dedup(D, ctx->seed_off_h[e], ctx->seed_off_h[e + 1], e, 1, (size_t)ctx->hit_off_h[e] + e,
-                      (size_t)(ctx->hit_off_h[e + 1] - ctx->hit_off_h[e]), st));
+                      (size_t)(ctx->hit_off_h[e + 1] - ctx->hit_off_h[e]), false, st));
   }
   ctx->deduped = true;
   return KF_OK;

@@ -268,9 +268,10 @@ size_t scan_tmp_elems(size_t n);
 size_t bin_group_elems(int n_events, int n_layers, int n_eta, int n_phi);
 // kf_dedup.cu
 // Tracks [t_begin, t_end), those of events [e_begin, e_begin + n_events), whose
-// list heads are head[head_begin, head_begin + n_heads).
+// list heads are head[head_begin, head_begin + n_heads).  clear_status: the
+// status word is zeroed first.
 cudaError_t launch_dedup(const DedupParams& P, int t_begin, int t_end, int e_begin, int n_events, size_t head_begin,
-                         size_t n_heads, cudaStream_t st);
+                         size_t n_heads, bool clear_status, cudaStream_t st);
 // Seed cleaning of the seeds at positions [pos_begin, pos_end) of the theta
 // order, which are those of events [e_begin, e_begin + n_events).
 cudaError_t launch_seed_clean(const SeedCleanParams& P, int pos_begin, int pos_end, int e_begin, int n_events,

@@ -51,3 +51,19 @@ def test_noalloc_lists_match_sequential_walk(n, L):
     ref = oracle.dedup(hits, n_found, chi2.astype(np.float64), float(np.float32(0.4)))
     ref = np.where(n_found > 0, ref, 0)
     assert np.array_equal(keep.cpu().numpy(), ref)
+
+
+def test_event_beyond_the_shared_memory_states():
+    """An event of more tracks than the resolution holds in shared memory."""
+    from kfhelp import tracker_for
+    from synth import make_batch
+    b = make_batch("c1b", tracks=25000)
+    t = tracker_for(b)
+    t.find_tracks()
+    t.remove_duplicates()
+    trk = t.get_tracks()
+    t.close()
+    assert b.n_seeds > 24576
+    ref = oracle.dedup(trk["hits"], trk["n_found"], trk["chi2"].astype(np.float64), 0.5)
+    assert np.array_equal(trk["keep"], ref)
+    assert 0 < b.n_seeds - int(ref.sum()) < b.n_seeds
