@@ -29,12 +29,11 @@
 // double precision across blocks).
 // The tracks of the fit's careful list (a crossing with cos(alpha) < 0.5, a
 // plane step along more than half a radian, or a loose prior) are reversed
-// by separate passes, which can run beside the FP32 pass after the fit's own
+// by a separate pass, which can run beside the FP32 pass after the fit's own
 // careful pass: those with a crossing below cos(alpha) = 0.2 or such a plane
-// step keep their adjoints in double and run those steps in double; the
-// others run the FP32 code.  The rest are reversed in FP32 from the
-// checkpoints.
-#include <type_traits>
+// step run those steps, and keep their adjoints between them, in double;
+// everything else runs the FP32 code, from the checkpoints.
+#include <algorithm>
 
 #include "kf_common.cuh"
 #include "kf_internal.h"
@@ -148,11 +147,10 @@ __device__ __forceinline__ void ksincos_acc(const Dir6<S>& a, Dir6<S>* s, Dir6<S
 namespace {
 
 constexpr float ADJ_CAREFUL_COS = ADJOINT_CAREFUL_COS;
-// Threads per block of the adjoint kernels; also the row stride (in floats)
-// of the segment buffer in shared memory.
+// Threads per block of the FP32 pass and of the careful pass; also the row
+// stride LD (in floats) of their columns in shared memory.
 constexpr int ADJ_THREADS = 128;
-constexpr int LD = ADJ_THREADS;
-static_assert((LD & (LD - 1)) == 0, "column rotation by a mask");
+constexpr int ADJ_CAREFUL_THREADS = 32;
 
 // Derivatives of f1 and f2 (the helix functions of kf_common.cuh) in psi:
 // f1' = -(sin psi + 2 f1)/psi, f2' = (cos psi - 2 f2)/psi, by the term-wise
@@ -1053,41 +1051,33 @@ __device__ __forceinline__ bool near_tangent(const DevGeom& g, const float (&p)[
   return cosa < ADJ_CAREFUL_COS;
 }
 
-// Forward step in precision S on float storage: the state before the step at
-// st[q * LD], q < 27; the state after it goes to st[(27 + q) * LD].
-template <class S, bool EL, bool DISK>
-__device__ __noinline__ void fwd_step_store(const DevGeom& g, float* st, const Hit<S>& h, bool first, bool last) {
-  S p[6], C[21];
-  for (int q = 0; q < 6; ++q) p[q] = (S)st[q * LD];
-  for (int q = 0; q < 21; ++q) C[q] = (S)st[(6 + q) * LD];
-  fwd_step<S, EL, DISK>(g, p, C, h, first, last);
-  for (int q = 0; q < 6; ++q) st[(27 + q) * LD] = (float)p[q];
-  for (int q = 0; q < 21; ++q) st[(27 + 6 + q) * LD] = (float)C[q];
+// Forward step (not a track's first) in double on float storage: the state
+// before it at in[q * LD], the state after it to out[q * LD].
+template <bool EL, bool DISK, int LD>
+__device__ __noinline__ void fwd_step_double(const DevGeom& g, const float* in, float* out, const Hit<double>& h,
+                                             bool last) {
+  double p[6], C[21];
+  for (int q = 0; q < 6; ++q) p[q] = (double)in[q * LD];
+  for (int q = 0; q < 21; ++q) C[q] = (double)in[(6 + q) * LD];
+  fwd_step<double, EL, DISK>(g, p, C, h, false, last);
+  for (int q = 0; q < 6; ++q) out[q * LD] = (float)p[q];
+  for (int q = 0; q < 21; ++q) out[(6 + q) * LD] = (float)C[q];
 }
 
-// Reverse step in precision S with the adjoints kept in A (double in the
-// careful pass, float otherwise); the state before the step at st[q * LD].
-template <class S, class A, bool EL, bool DISK>
-__device__ __noinline__ void rev_step_store(const DevGeom& g, const float* st, const Hit<S>& h, bool first,
-                                            bool last, A (&pbA)[6], A (&CbA)[6][6], A (&hbA)[3]) {
-  S p[6], C[21], pb[6], Cb[6][6], hb[3];
-  for (int q = 0; q < 6; ++q) p[q] = (S)st[q * LD];
-  for (int q = 0; q < 21; ++q) C[q] = (S)st[(6 + q) * LD];
-  for (int i = 0; i < 6; ++i) {
-    pb[i] = (S)pbA[i];
-    for (int j = 0; j < 6; ++j) Cb[i][j] = (S)CbA[i][j];
-  }
-  rev_step<S, EL, DISK>(g, p, C, h, first, last, pb, Cb, hb);
-  for (int i = 0; i < 6; ++i) {
-    pbA[i] = (A)pb[i];
-    for (int j = 0; j < 6; ++j) CbA[i][j] = (A)Cb[i][j];
-  }
-  for (int i = 0; i < 3; ++i) hbA[i] = (A)hb[i];
+// Reverse step in double with its adjoints in local memory; the state before
+// the step at st[q * LD].
+template <bool EL, bool DISK, int LD>
+__device__ __noinline__ void rev_step_double(const DevGeom& g, const float* st, const Hit<double>& h, bool first,
+                                             bool last, double (&pb)[6], double (&Cb)[6][6], double (&hb)[3]) {
+  double p[6], C[21];
+  for (int q = 0; q < 6; ++q) p[q] = (double)st[q * LD];
+  for (int q = 0; q < 21; ++q) C[q] = (double)st[(6 + q) * LD];
+  rev_step<double, EL, DISK>(g, p, C, h, first, last, pb, Cb, hb);
 }
 
 // Forward step of the FP32 pass, inlined (as rev_step_regs): the state
 // before it at in[q * LD], the state after it to out[q * LD].
-template <bool EL, bool DISK>
+template <bool EL, bool DISK, int LD>
 __device__ __forceinline__ void fwd_step_regs(const DevGeom& g, const float* in, float* out, const Hit<float>& h,
                                               bool first, bool last) {
   float p[6], C[21];
@@ -1105,7 +1095,7 @@ __device__ __forceinline__ void fwd_step_regs(const DevGeom& g, const float* in,
 // The same reverse step inlined into the FP32 pass, so that the adjoints stay
 // in registers (an out-of-line call takes them by reference, through local
 // memory).
-template <bool EL, bool DISK>
+template <bool EL, bool DISK, int LD>
 __device__ __forceinline__ void rev_step_regs(const DevGeom& g, const float* st, const Hit<float>& h, bool first,
                                               bool last, float (&pb)[6], float (&Cb)[6][6], float (&hb)[3]) {
   float p[6], C[21];
@@ -1114,84 +1104,6 @@ __device__ __forceinline__ void rev_step_regs(const DevGeom& g, const float* st,
 #pragma unroll
   for (int q = 0; q < 21; ++q) C[q] = st[(6 + q) * LD];
   rev_step<float, EL, DISK>(g, p, C, h, first, last, pb, Cb, hb);
-}
-
-// Reverse sweep of the track at position i of the fit's order, from the
-// fit's checkpoints (column i).  CAREFUL:
-// the track the fit flagged as near-tangent; its near-tangent steps run in
-// double precision and its adjoints are kept in double.  seg: this thread's
-// column of the block's segment buffer in shared memory (states before each
-// step of a segment, [slot][27][LD]).
-template <bool CAREFUL, bool EL, bool DISK>
-__device__ void adjoint_track(const AdjParams& P, int i, float* seg) {
-  using A = typename std::conditional<CAREFUL, double, float>::type;
-  const DevGeom& g = P.g;
-  const int t = P.order[i];  // the track at position i of the fit's order (checkpoint column i)
-  static_assert(CAREFUL, "the FP32 pass is adjoint_track_fp32");
-  if (P.fit_status[t] != KF_FIT_OK) {
-    if (P.g_seed)
-      for (int k = 0; k < 6; ++k) P.g_seed[(size_t)k * P.ns + t] = 0.f;
-    return;
-  }
-  const int n = P.n_list[t];
-  const int* lst = P.lists + (size_t)t * P.max_len;
-  const int hoff = P.hit_off[P.seed_event[t]];
-  const int stride = P.stride;
-  A pb[6], Cb[6][6];
-  for (int i = 0; i < 6; ++i) {
-    pb[i] = A(0);
-    for (int j = 0; j < 6; ++j) Cb[i][j] = A(0);
-  }
-  for (int c = (n - 1) / stride; c >= 0; --c) {
-    const int k0 = c * stride, k1 = min(n, k0 + stride);
-    const float* ck = P.ckpt + (size_t)c * 27 * P.ns + i;
-    for (int q = 0; q < 27; ++q) seg[q * LD] = ck[(size_t)q * P.ns];
-    for (int k = k0; k + 1 < k1; ++k) {
-      float* st = seg + (k - k0) * 27 * LD;
-      const int hi = hoff + lst[k];
-      if (CAREFUL && k > 0) {
-        float pf[6];
-        for (int q = 0; q < 6; ++q) pf[q] = st[q * LD];
-        const int Lh = P.hlayer[hi];
-        if (is_disk(g, Lh) ? plane_careful(g, pf, plane_z(g, Lh)) : near_tangent(g, pf, g.radius[Lh])) {
-          fwd_step_store<double, EL, DISK>(g, st, load_hit<double>(P, hi), k == 0, k + 1 == n);
-          continue;
-        }
-      }
-      fwd_step_store<float, EL, DISK>(g, st, load_hit<float>(P, hi), k == 0, k + 1 == n);
-    }
-    for (int k = k1 - 1; k >= k0; --k) {
-      const float* st = seg + (k - k0) * 27 * LD;
-      const int hl = lst[k];
-      const int hi = hoff + hl;
-      A hb[3];
-      bool dbl = false;
-      if (CAREFUL && k > 0) {
-        float pf[6];
-        for (int q = 0; q < 6; ++q) pf[q] = st[q * LD];
-        const int Lh = P.hlayer[hi];
-        dbl = is_disk(g, Lh) ? plane_careful(g, pf, plane_z(g, Lh)) : near_tangent(g, pf, g.radius[Lh]);
-      }
-      if (dbl)
-        rev_step_store<double, A, EL, DISK>(g, st, load_hit<double>(P, hi), k == 0, k + 1 == n, pb, Cb, hb);
-      else
-        rev_step_store<float, A, EL, DISK>(g, st, load_hit<float>(P, hi), k == 0, k + 1 == n, pb, Cb, hb);
-      float* gh = P.g_hits + 3 * (size_t)hi;  // a hit can be on several tracks
-      atomicAdd(gh + 0, (float)hb[0]);
-      atomicAdd(gh + 1, (float)hb[1]);
-      atomicAdd(gh + 2, (float)hb[2]);
-      // the layer's alignment gradient (linear in the hit gradient; few
-      // tracks); disks carry no alignment
-      const int L = P.hlayer[hi];
-      if (!is_disk(g, L)) {
-        atomicAdd(P.g_align_acc + 2 * L, -((double)P.hx[hi] * hb[1] - (double)P.hy[hi] * hb[0]) / g.radius[L]);
-        atomicAdd(P.g_align_acc + 2 * L + 1, -(double)hb[2]);
-      }
-    }
-  }
-  if (P.g_seed) {
-    for (int k = 0; k < 6; ++k) P.g_seed[(size_t)k * P.ns + t] = (float)pb[k];
-  }
 }
 
 // Asynchronous copy of one 4-byte word from global memory to this thread's
@@ -1203,25 +1115,39 @@ __device__ __forceinline__ void cp_async4(float* sdst, const void* gsrc) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
-// Shared memory of the FP32 pass, in floats per thread column (LD apart):
+// Shared memory of the passes, in floats per thread column (LD apart):
 //   seg [stride - 1][27]  states before a segment's steps after its first
 //   ckb [2][27]           the segment's checkpoint (two buffers, by parity)
 //   hbf [2][stride][5]    its hits: x, y, z, layer and event-global index (int bits)
 //   lbf [2][stride]       event-local hit indices of a later segment
 __host__ __device__ constexpr int fp32_col_floats(int stride) { return 27 * (stride - 1) + 54 + 12 * stride; }
 
-// Reverse sweep of the track at position i of the fit's order in FP32 (the
-// tracks the fit left without a crossing below ADJ_CAREFUL_COS).  Segment c-1's
-// checkpoint and hits are copied into shared memory while segment c is
-// reversed, and segment c-2's hit indices with them, so that a segment's
-// steps wait on no global load.  col: this thread's column; s_al, s_R: the
-// layers' alignment and radii in shared memory; ga: this thread's column of
-// alignment-gradient sums (rows 2L and 2L + 1: layer L's rotation and z).
-// listed: the track comes from the fit's careful list (else careful tracks
-// are skipped: the careful passes take them).
-template <bool EL, bool DISK>
-__device__ void adjoint_track_fp32(const AdjParams& P, int i, float* col, const float4* s_al, const float* s_R,
-                                   float* ga, bool listed) {
+// Whether step k of a track (state before it at st[q * LD], its hit on surface
+// L) runs in double in the careful pass.
+template <bool DISK, int LD>
+__device__ __forceinline__ bool double_step(const DevGeom& g, const float* st, int L) {
+  float p[6];
+#pragma unroll
+  for (int q = 0; q < 6; ++q) p[q] = st[q * LD];
+  return DISK && is_disk(g, L) ? plane_careful(g, p, plane_z(g, L)) : near_tangent(g, p, g.radius[L]);
+}
+
+// Reverse sweep of the track at position i of the fit's order in FP32, from
+// the fit's checkpoints (column i).  Segment c-1's checkpoint and hits are
+// copied into shared memory while segment c is reversed, and segment c-2's hit
+// indices with them, so that a segment's steps wait on no global load.  col:
+// this thread's column; s_al, s_R: the layers' alignment and radii in shared
+// memory; ga: this thread's column of alignment-gradient sums (rows 2L and 2L
+// + 1: layer L's rotation and z).  listed: the track comes from the fit's
+// careful list (else careful tracks are skipped: the careful pass takes them).
+// DBL: a track with near-tangent steps (cos below ADJ_CAREFUL_COS, or a long
+// plane step).  Those run in double, their adjoints in double from one to the
+// next; they lie at the end of the track, at or after the step at which the
+// fit's FP32 pass stopped it, so the sweep begins with them and goes on in
+// FP32.  Its alignment sums are formed in double (s_Ri: 1/R).
+template <bool EL, bool DISK, int LD, bool DBL>
+__device__ void adjoint_track(const AdjParams& P, int i, float* col, const float4* s_al, const float* s_R, float* ga,
+                              bool listed, const double* s_Ri = nullptr) {
   const DevGeom& g = P.g;
   const int t = P.order[i];
   if (!listed && P.careful_flag[t]) return;  // the careful passes', which run beside this one
@@ -1267,6 +1193,11 @@ __device__ void adjoint_track_fp32(const AdjParams& P, int i, float* col, const 
 #pragma unroll
     for (int b = 0; b < 6; ++b) Cb[a][b] = 0.f;
   }
+  // DBL: the first step that can run in double (the flag holds the step the
+  // fit's FP32 pass stopped at, plus one), and the adjoints while in double
+  const int k_dbl = DBL ? max((int)P.careful_flag[t] - 1, 1) : 0;
+  double pbd[6], Cbd[6][6];
+  bool in_dbl = false;
   const int last = (n - 1) / stride;
   seg_lists(last);
   cp_async_commit();
@@ -1308,15 +1239,48 @@ __device__ void adjoint_track_fp32(const AdjParams& P, int i, float* col, const 
       return h;
     };
     // state before step k: the checkpoint for k0, else seg slot k - k0 - 1
-    for (int k = k0; k + 1 < k1; ++k)
-      fwd_step_regs<EL, DISK>(g, k == k0 ? ck : seg + (k - k0 - 1) * 27 * LD, seg + (k - k0) * 27 * LD,
-                              hit_of(k), k == 0, k + 1 == n);
+    for (int k = k0; k + 1 < k1; ++k) {
+      const float* st = k == k0 ? ck : seg + (k - k0 - 1) * 27 * LD;
+      float* out = seg + (k - k0) * 27 * LD;
+      if constexpr (DBL) {
+        if (k >= k_dbl && double_step<DISK, LD>(g, st, __float_as_int(hs[((k - k0) * 5 + 3) * LD]))) {
+          fwd_step_double<EL, DISK, LD>(g, st, out, load_hit<double>(P, __float_as_int(hs[((k - k0) * 5 + 4) * LD])),
+                                        k + 1 == n);
+          continue;
+        }
+      }
+      fwd_step_regs<EL, DISK, LD>(g, st, out, hit_of(k), k == 0, k + 1 == n);
+    }
     for (int k = k1 - 1; k >= k0; --k) {
-      float hb[3];
-      rev_step_regs<EL, DISK>(g, k == k0 ? ck : seg + (k - k0 - 1) * 27 * LD, hit_of(k), k == 0, k + 1 == n, pb, Cb,
-                              hb);
+      const float* st = k == k0 ? ck : seg + (k - k0 - 1) * 27 * LD;
       const float* hd = hs + (k - k0) * 5 * LD;
       const int hi = __float_as_int(hd[4 * LD]);
+      float hb[3];
+      double hbd[3];
+      bool dbl = false;
+      if constexpr (DBL) {
+        dbl = k >= k_dbl && double_step<DISK, LD>(g, st, __float_as_int(hd[3 * LD]));
+        if (dbl) {
+          if (!in_dbl)
+            for (int a = 0; a < 6; ++a) {
+              pbd[a] = pb[a];
+              for (int b = 0; b < 6; ++b) Cbd[a][b] = Cb[a][b];
+            }
+          in_dbl = true;
+          rev_step_double<EL, DISK, LD>(g, st, load_hit<double>(P, hi), false, k + 1 == n, pbd, Cbd, hbd);
+#pragma unroll
+          for (int a = 0; a < 3; ++a) hb[a] = (float)hbd[a];
+        } else if (in_dbl) {
+          in_dbl = false;
+#pragma unroll
+          for (int a = 0; a < 6; ++a) {
+            pb[a] = (float)pbd[a];
+#pragma unroll
+            for (int b = 0; b < 6; ++b) Cb[a][b] = (float)Cbd[a][b];
+          }
+        }
+      }
+      if (!DBL || !dbl) rev_step_regs<EL, DISK, LD>(g, st, hit_of(k), k == 0, k + 1 == n, pb, Cb, hb);
       float* gh = P.g_hits + 3 * (size_t)hi;  // a hit can be on several tracks
       atomicAdd(gh + 0, hb[0]);
       atomicAdd(gh + 1, hb[1]);
@@ -1324,68 +1288,123 @@ __device__ void adjoint_track_fp32(const AdjParams& P, int i, float* col, const 
       // the layer's alignment gradient (linear in the hit gradient), summed
       // in this thread's column
       const int L = __float_as_int(hd[3 * LD]);
-      if (!DISK || !is_disk(g, L)) {
+      if (DBL && !(DISK && is_disk(g, L))) {
+        if (!dbl) {
+#pragma unroll
+          for (int a = 0; a < 3; ++a) hbd[a] = hb[a];
+        }
+        atomicAdd(P.g_align_acc + 2 * L, -((double)hd[0] * hbd[1] - (double)hd[LD] * hbd[0]) * s_Ri[L]);
+        atomicAdd(P.g_align_acc + 2 * L + 1, -hbd[2]);
+      } else if (!DISK || !is_disk(g, L)) {
         ga[2 * L * LD] -= kfma(hd[0], hb[1], -hd[LD] * hb[0]) / s_R[L];
         ga[(2 * L + 1) * LD] -= hb[2];
       }
     }
   }
   if (P.g_seed) {
-    for (int k = 0; k < 6; ++k) P.g_seed[(size_t)k * P.ns + t] = pb[k];
+    for (int k = 0; k < 6; ++k) P.g_seed[(size_t)k * P.ns + t] = DBL && in_dbl ? (float)pbd[k] : pb[k];
   }
 }
 
-// Passes of the adjoint: the FP32 pass over every position (the tracks of
-// the fit's careful list skipped), and over the careful list the entries
-// without CAREFUL_DBL_BIT in FP32 and those with it in double.
-enum { ADJ_ALL = 0, ADJ_LIST_FP32 = 1, ADJ_LIST_DBL = 2 };
+// Common part of the passes: the layers' alignment and radii and the columns
+// of alignment sums in shared memory; returns the sums' first row.
+template <int LD>
+__device__ __forceinline__ float* adjoint_shared(const AdjParams& P, float* cols, float4* s_al, float* s_R) {
+  const int nga = 2 * P.g.n_layers;
+  float* const ga_all = cols + (size_t)fp32_col_floats(P.stride) * LD;  // [nga][LD]
+  for (int q = 0; q < nga; ++q) ga_all[q * LD + threadIdx.x] = 0.f;
+  for (int l = threadIdx.x; l < P.g.n_layers; l += LD) {
+    const Align4 a = P.align[l];
+    s_al[l] = make_float4(a.ca, a.sa, a.dphi, a.az);
+    s_R[l] = P.g.radius[l];
+  }
+  __syncthreads();
+  return ga_all;
+}
+template <int LD>
+__device__ __forceinline__ void adjoint_sums(const AdjParams& P, const float* ga_all) {
+  static_assert((LD & (LD - 1)) == 0, "column rotation by a mask");
+  __syncthreads();
+  for (int q = threadIdx.x; q < 2 * P.g.n_layers; q += LD) {  // row q over the columns, rotated by q (banks)
+    float a = 0.f;
+    for (int c = 0; c < LD; ++c) a += ga_all[q * LD + ((c + q) & (LD - 1))];
+    if (a != 0.f) atomicAdd(P.g_align_acc + q, (double)a);
+  }
+}
 
-template <int MODE, bool EL, bool DISK = false>
+// FP32 pass over every position (the tracks of the fit's careful list skipped).
+template <bool EL, bool DISK>
 __global__ void __launch_bounds__(ADJ_THREADS) k_adjoint(const AdjParams P) {
-  // double pass: [stride][27][LD]; FP32 passes: columns of fp32_col_floats,
-  // then 2 x layers rows of alignment-gradient sums
-  extern __shared__ float seg_all[];
-  float* seg = seg_all + threadIdx.x;
-  if constexpr (MODE != ADJ_LIST_DBL) {
-    __shared__ float4 s_al[KF_MAX_LAYERS];
-    __shared__ float s_R[KF_MAX_LAYERS];
-    const int nga = 2 * P.g.n_layers;
-    float* const ga_all = seg_all + (size_t)fp32_col_floats(P.stride) * LD;  // [nga][LD]
-    float* const ga = ga_all + threadIdx.x;
-    for (int q = 0; q < nga; ++q) ga[q * LD] = 0.f;
-    for (int l = threadIdx.x; l < P.g.n_layers; l += blockDim.x) {
-      const Align4 a = P.align[l];
-      s_al[l] = make_float4(a.ca, a.sa, a.dphi, a.az);
-      s_R[l] = P.g.radius[l];
-    }
-    __syncthreads();
-    if constexpr (MODE == ADJ_ALL) {
-      const int i = blockIdx.x * blockDim.x + threadIdx.x;
-      if (i < P.ns) adjoint_track_fp32<EL, DISK>(P, i, seg, s_al, s_R, ga, false);
-    } else {
-      const unsigned n = *P.careful_count;
-      for (unsigned j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+  extern __shared__ float cols[];  // columns of fp32_col_floats, then 2 x layers rows of alignment sums
+  __shared__ float4 s_al[KF_MAX_LAYERS];
+  __shared__ float s_R[KF_MAX_LAYERS];
+  float* const ga_all = adjoint_shared<ADJ_THREADS>(P, cols, s_al, s_R);
+  const int i = blockIdx.x * ADJ_THREADS + threadIdx.x;
+  if (i < P.ns)
+    adjoint_track<EL, DISK, ADJ_THREADS, false>(P, i, cols + threadIdx.x, s_al, s_R, ga_all + threadIdx.x, false);
+  adjoint_sums<ADJ_THREADS>(P, ga_all);
+}
+
+// Careful passes, one warp per block, over the tracks with double-precision
+// steps (DBL) and over the rest of the careful list, each list dealt evenly to
+// the blocks (as k_fit_careful's: with few tracks, one per warp).  A double
+// step is bound by its unit, 64 clocks per warp instruction; a track has one
+// to three of them, and everything else of it runs in the FP32 code.  The two
+// passes are kernels of their own, beside each other: the double steps' code
+// would cost the FP32 one 96 registers.
+template <bool EL, bool DISK, bool DBL>
+__global__ void __launch_bounds__(ADJ_CAREFUL_THREADS) k_adjoint_careful(const AdjParams P) {
+  extern __shared__ float cols[];
+  __shared__ float4 s_al[KF_MAX_LAYERS];
+  __shared__ float s_R[KF_MAX_LAYERS];
+  __shared__ double s_Ri[DBL ? KF_MAX_LAYERS : 1];
+  constexpr int T = ADJ_CAREFUL_THREADS;
+  const unsigned n = DBL ? *P.dbl_count : *P.careful_count;
+  const unsigned per = min((unsigned)T, (n + gridDim.x - 1) / gridDim.x);  // tracks per warp and round
+  if (blockIdx.x * per >= n) return;
+  if constexpr (DBL)
+    for (int l = threadIdx.x; l < P.g.n_layers; l += T) s_Ri[l] = 1.0 / (double)P.g.radius[l];
+  float* const ga_all = adjoint_shared<T>(P, cols, s_al, s_R);
+  if (threadIdx.x < per) {
+    for (unsigned j = blockIdx.x * per + threadIdx.x; j < n; j += gridDim.x * per) {
+      if constexpr (DBL) {
+        adjoint_track<EL, DISK, T, true>(P, P.dbl_list[j], cols + threadIdx.x, s_al, s_R, nullptr, true, s_Ri);
+      } else {
         const unsigned v = (unsigned)P.careful_list[j];
-        if (!(v & CAREFUL_DBL_BIT)) adjoint_track_fp32<EL, DISK>(P, (int)v, seg, s_al, s_R, ga, true);
+        if (!(v & CAREFUL_DBL_BIT))
+          adjoint_track<EL, DISK, T, false>(P, (int)v, cols + threadIdx.x, s_al, s_R, ga_all + threadIdx.x, true);
       }
     }
-    __syncthreads();
-    for (int q = threadIdx.x; q < nga; q += blockDim.x) {  // row q over the columns, rotated by q (banks)
-      float a = 0.f;
-      for (int c = 0; c < LD; ++c) a += ga_all[q * LD + ((c + q) & (LD - 1))];
-      if (a != 0.f) atomicAdd(P.g_align_acc + q, (double)a);
-    }
-  } else {  // packed list: the first blocks take all of them and the others end at once
-    const unsigned n = *P.dbl_count;
-    for (unsigned j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x)
-      adjoint_track<true, EL, DISK>(P, P.dbl_list[j], seg);
   }
+  if constexpr (!DBL) adjoint_sums<T>(P, ga_all);
 }
 
 __global__ void k_adjoint_finish(const AdjParams P) {
   const int i = threadIdx.x;
   if (i < 2 * P.g.n_layers) P.g_align[i] = (float)P.g_align_acc[i];
 }
+
+}  // namespace
+
+namespace {
+
+typedef void (*Kernel)(AdjParams);
+// The kernel of a pass for a detector (energy loss on any surface, endcap disks).
+template <bool EL, bool DISK>
+Kernel kernel_t(int pass) {
+  return pass == ADJ_MAIN ? k_adjoint<EL, DISK>
+                          : pass == ADJ_LIST ? k_adjoint_careful<EL, DISK, false> : k_adjoint_careful<EL, DISK, true>;
+}
+Kernel kernel_of(const AdjParams& P, int pass) {
+  bool el = P.g.n_disks > 0 && P.g.disk_eloss > 0.f;
+  for (int l = 0; l < P.g.n_layers; ++l) el = el || P.g.eloss[l] > 0.f;
+  if (P.g.n_disks > 0) return el ? kernel_t<true, true>(pass) : kernel_t<false, true>(pass);
+  return el ? kernel_t<true, false>(pass) : kernel_t<false, false>(pass);
+}
+size_t smem_bytes(const AdjParams& P, int threads) {
+  return sizeof(float) * (fp32_col_floats(P.stride) + 2 * P.g.n_layers) * (size_t)threads;
+}
+constexpr int ADJ_CAREFUL_BLOCKS = 152;  // one per SM
 
 }  // namespace
 
@@ -1398,52 +1417,25 @@ cudaError_t launch_adjoint_begin(const AdjParams& P, cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(P.g_align_acc, 0, sizeof(double) * 2 * KF_MAX_LAYERS, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(P.g_hits, 0, sizeof(float) * 3 * (size_t)P.n_hits, st);
   if (e != cudaSuccess) return e;
-  const int smem_c = (int)(sizeof(float) * 27 * (size_t)P.stride * ADJ_THREADS);
-  const int smem_f = (int)(sizeof(float) * (fp32_col_floats(P.stride) + 2 * P.g.n_layers) * (size_t)ADJ_THREADS);
-  const void* fns[12] = {(const void*)k_adjoint<ADJ_ALL, false>,        (const void*)k_adjoint<ADJ_LIST_FP32, false>,
-                         (const void*)k_adjoint<ADJ_LIST_DBL, false>,   (const void*)k_adjoint<ADJ_ALL, true>,
-                         (const void*)k_adjoint<ADJ_LIST_FP32, true>,   (const void*)k_adjoint<ADJ_LIST_DBL, true>,
-                         (const void*)k_adjoint<ADJ_ALL, false, true>,  (const void*)k_adjoint<ADJ_LIST_FP32, false, true>,
-                         (const void*)k_adjoint<ADJ_LIST_DBL, false, true>, (const void*)k_adjoint<ADJ_ALL, true, true>,
-                         (const void*)k_adjoint<ADJ_LIST_FP32, true, true>, (const void*)k_adjoint<ADJ_LIST_DBL, true, true>};
-  for (int k = 0; k < 12 && e == cudaSuccess; ++k)
-    e = cudaFuncSetAttribute(fns[k], cudaFuncAttributeMaxDynamicSharedMemorySize, k % 3 == 2 ? smem_c : smem_f);
+  for (int pass = 0; pass < 3 && e == cudaSuccess; ++pass)
+    e = cudaFuncSetAttribute((const void*)kernel_of(P, pass), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)smem_bytes(P, pass == ADJ_MAIN ? ADJ_THREADS : ADJ_CAREFUL_THREADS));
   return e;
 }
 
-cudaError_t launch_adjoint_pass(const AdjParams& P, bool careful, cudaStream_t st) {
+cudaError_t launch_adjoint_pass(const AdjParams& P, int pass, cudaStream_t st) {
   if (P.ns <= 0) return cudaSuccess;
-  const size_t smem_c = sizeof(float) * 27 * (size_t)P.stride * ADJ_THREADS;
-  const size_t smem_f = sizeof(float) * (fp32_col_floats(P.stride) + 2 * P.g.n_layers) * (size_t)ADJ_THREADS;
-  bool el = false;  // energy loss on any layer: the variant with its code
-  for (int l = 0; l < P.g.n_layers; ++l) el = el || P.g.eloss[l] > 0.f;
-  const int grid_all = (P.ns + ADJ_THREADS - 1) / ADJ_THREADS;
-  // flagged tracks are a few percent: a grid for a twentieth of all, striding
-  // over however many there are
-  const int grid_careful = (P.ns / 20 + ADJ_THREADS - 1) / ADJ_THREADS + 1;
-  // the double pass: blocks of 32 threads (its tracks' double-precision
-  // steps are bound by the SM's FP64 rate, so they spread over many SMs)
-  constexpr int DBL_THREADS = 32;
-  const int grid_dbl = (P.ns / 20 + DBL_THREADS - 1) / DBL_THREADS + 1;
-  if (P.g.n_disks > 0) {  // the disk variants; energy loss on a layer or on the disks
-    if (P.g.disk_eloss > 0.f) el = true;
-    if (!careful) {
-      if (el) k_adjoint<ADJ_ALL, true, true><<<grid_all, ADJ_THREADS, smem_f, st>>>(P);
-      else k_adjoint<ADJ_ALL, false, true><<<grid_all, ADJ_THREADS, smem_f, st>>>(P);
-    } else {
-      if (el) k_adjoint<ADJ_LIST_DBL, true, true><<<grid_dbl, DBL_THREADS, smem_c, st>>>(P);
-      else k_adjoint<ADJ_LIST_DBL, false, true><<<grid_dbl, DBL_THREADS, smem_c, st>>>(P);
-      if (el) k_adjoint<ADJ_LIST_FP32, true, true><<<grid_careful, ADJ_THREADS, smem_f, st>>>(P);
-      else k_adjoint<ADJ_LIST_FP32, false, true><<<grid_careful, ADJ_THREADS, smem_f, st>>>(P);
-    }
-  } else if (!careful) {
-    if (el) k_adjoint<ADJ_ALL, true><<<grid_all, ADJ_THREADS, smem_f, st>>>(P);
-    else k_adjoint<ADJ_ALL, false><<<grid_all, ADJ_THREADS, smem_f, st>>>(P);
-  } else {  // the careful list: its tracks with double steps, then the others
-    if (el) k_adjoint<ADJ_LIST_DBL, true><<<grid_dbl, DBL_THREADS, smem_c, st>>>(P);
-    else k_adjoint<ADJ_LIST_DBL, false><<<grid_dbl, DBL_THREADS, smem_c, st>>>(P);
-    if (el) k_adjoint<ADJ_LIST_FP32, true><<<grid_careful, ADJ_THREADS, smem_f, st>>>(P);
-    else k_adjoint<ADJ_LIST_FP32, false><<<grid_careful, ADJ_THREADS, smem_f, st>>>(P);
+  const Kernel k = kernel_of(P, pass);
+  if (pass == ADJ_MAIN) {
+    k<<<(P.ns + ADJ_THREADS - 1) / ADJ_THREADS, ADJ_THREADS, smem_bytes(P, ADJ_THREADS), st>>>(P);
+  } else {
+    // about a 64th of all tracks are flagged, a 350th have double steps: grids
+    // for those at 32 per block, so that a large batch packs its warps, and at
+    // least one block per SM, so that a small one spreads its tracks (of a
+    // single track each up to 10,000 tracks); striding over however many there are
+    const int of = (pass == ADJ_LIST ? 64 : 350) * ADJ_CAREFUL_THREADS;
+    const int grid = std::max(P.ns / of + 1, std::min(P.ns, ADJ_CAREFUL_BLOCKS));
+    k<<<grid, ADJ_CAREFUL_THREADS, smem_bytes(P, ADJ_CAREFUL_THREADS), st>>>(P);
   }
   return cudaGetLastError();
 }

@@ -65,9 +65,10 @@ struct kf_ctx {
   int graph_n_seeds = -1;
   int stage_timing = 0;
   cudaEvent_t ev[12] = {};  // start/end of bin, find, dedup, fit, adjoint, seed cleaning
-  // Side stream (highest priority) for the careful passes that run beside
-  // the main passes; fork/join events.
-  cudaStream_t side = nullptr;
+  // Side streams for the careful passes that run beside the main passes: side
+  // (highest priority) for the long double-precision chains, side2 (lowest)
+  // for work that fills what the main pass leaves; fork/join events.
+  cudaStream_t side = nullptr, side2 = nullptr;
   // Inside a graph capture with the adjoint: kf_fit_tracks leaves the fit's
   // careful pass to kf_fit_adjoint, which runs it on the side stream before
   // the careful adjoint, beside the FP32 adjoint (which needs neither).
@@ -76,7 +77,7 @@ struct kf_ctx {
   // FP32 pass fits every found track; the caller then clears the removed ones)
   // and always leaves its careful pass for later.
   bool fit_beside_dedup = false;
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_fork2 = nullptr, ev_join2 = nullptr;
   std::string err = "";
 };
 
@@ -345,8 +346,9 @@ int kf_create(const kf_detector* det, const kf_config* cfg, kf_ctx** out) {
     int least = 0, greatest = 0;
     e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&ctx->side, cudaStreamNonBlocking, greatest);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&ctx->side2, cudaStreamNonBlocking, least);
+    for (cudaEvent_t* ev : {&ctx->ev_fork, &ctx->ev_join, &ctx->ev_fork2, &ctx->ev_join2})
+      if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
   }
   if (e == cudaSuccess) e = grow(ctx->counters, 8 * KF_N_COUNTERS);
   if (e == cudaSuccess) e = grow(ctx->status, 64);
@@ -384,9 +386,10 @@ int kf_destroy(kf_ctx* ctx) {
   if (!ctx) return KF_ERR_ARG;
   for (cudaEvent_t& e : ctx->ev)
     if (e) cudaEventDestroy(e);
-  if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
-  if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
-  if (ctx->side) cudaStreamDestroy(ctx->side);
+  for (cudaEvent_t e : {ctx->ev_fork, ctx->ev_join, ctx->ev_fork2, ctx->ev_join2})
+    if (e) cudaEventDestroy(e);
+  for (cudaStream_t s : {ctx->side, ctx->side2})
+    if (s) cudaStreamDestroy(s);
   if (ctx->exec) cudaGraphExecDestroy(ctx->exec);
   if (ctx->graph) cudaGraphDestroy(ctx->graph);
   for (DevBuf* b : all_bufs(ctx)) release(*b);
@@ -603,16 +606,13 @@ static void stage_mark(kf_ctx* ctx, int i, cudaStream_t st) {
 // Work on ctx->side after everything enqueued so far on st (fork), and st
 // after everything enqueued on ctx->side (join).  Inside a stream capture the
 // side stream joins the capture and becomes a parallel branch of the graph.
-static cudaError_t fork_side(kf_ctx* ctx, cudaStream_t st) {
-  cudaError_t e = cudaEventRecord(ctx->ev_fork, st);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0);
+static cudaError_t after(cudaStream_t to, cudaStream_t from, cudaEvent_t ev) {
+  cudaError_t e = cudaEventRecord(ev, from);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(to, ev, 0);
   return e;
 }
-static cudaError_t join_side(kf_ctx* ctx, cudaStream_t st) {
-  cudaError_t e = cudaEventRecord(ctx->ev_join, ctx->side);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ctx->ev_join, 0);
-  return e;
-}
+static cudaError_t fork_side(kf_ctx* ctx, cudaStream_t st) { return after(ctx->side, st, ctx->ev_fork); }
+static cudaError_t join_side(kf_ctx* ctx, cudaStream_t st) { return after(st, ctx->side, ctx->ev_join); }
 
 static FindParams find_params(kf_ctx* ctx) {
   FindParams P;
@@ -971,13 +971,17 @@ int kf_fit_adjoint(kf_ctx* ctx, float* g_align, float* g_hits, float* g_seed, in
   stage_mark(ctx, 8, st);
   CK(launch_adjoint_begin(A, st));
   CK(fork_side(ctx, st));
-  // the careful tracks beside the FP32 pass: their fit (if still to run),
-  // then their adjoint
+  // the careful tracks beside the FP32 pass: their fit (if still to run), then
+  // the adjoints of those with and without double-precision steps beside each
+  // other
   if (ctx->careful_fit_pending) CK(launch_fit_careful(F, ctx->side));
   ctx->careful_fit_pending = false;
-  CK(launch_adjoint_pass(A, true, ctx->side));
-  CK(launch_adjoint_pass(A, false, st));
+  CK(after(ctx->side2, ctx->side, ctx->ev_fork2));
+  CK(launch_adjoint_pass(A, ADJ_DBL, ctx->side));
+  CK(launch_adjoint_pass(A, ADJ_LIST, ctx->side2));
+  CK(launch_adjoint_pass(A, ADJ_MAIN, st));
   CK(join_side(ctx, st));
+  CK(after(st, ctx->side2, ctx->ev_join2));
   CK(launch_adjoint_end(A, st));
   stage_mark(ctx, 9, st);
   if (!device_ptrs) {

@@ -25,7 +25,7 @@ namespace {
 
 constexpr float CAREFUL_COS = 0.5f;
 constexpr int FIT_THREADS = 128;  // threads per block of the FP32 pass
-constexpr int CAREFUL_BLOCKS = 608;  // careful pass: four warps per SM
+constexpr int CAREFUL_BLOCKS = 304;  // careful pass: two warps per SM
 
 // One Kalman step on an endcap disk in scalar type T (the plane, the (r-phi, r)
 // measurement, the disk's scattering and loss).
@@ -147,7 +147,7 @@ __device__ __forceinline__ void leave_to_careful(const FitParams& P, int i, int 
   P.fit_chi2[t] = chi2;
   P.fit_status[t] = k;
   P.careful_list[atomicAdd(P.careful_count, 1u)] = i;
-  if (P.careful_flag) P.careful_flag[t] = 1;
+  if (P.careful_flag) P.careful_flag[t] = (unsigned char)min(k + 1, 255);
 }
 
 // Track at position i of the fit's order; checkpoints go to column i.
@@ -329,11 +329,11 @@ cudaError_t launch_fit_main(const FitParams& P, cudaStream_t st) {
 
 cudaError_t launch_fit_careful(const FitParams& P, cudaStream_t st) {
   if (P.ns <= 0) return cudaSuccess;
-  // flagged tracks are a few percent of all: a grid for a twentieth of them
-  // at 32 per block, at least CAREFUL_BLOCKS blocks (of a single track each
-  // in a small batch), striding over however many there are
+  // about a 64th of all tracks are flagged: a grid for them at 32 per block,
+  // at least CAREFUL_BLOCKS blocks (of a few tracks each in a small batch),
+  // striding over however many there are
   const int threads = 32;
-  const int careful_blocks = std::max((P.ns / 20 + threads - 1) / threads + 1, std::min(P.ns, CAREFUL_BLOCKS));
+  const int careful_blocks = std::max(P.ns / (64 * threads) + 1, std::min(P.ns, CAREFUL_BLOCKS));
   cudaError_t e = cudaMemsetAsync(P.dbl_count, 0, sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
   if (P.g.n_disks > 0) k_fit_careful<true><<<careful_blocks, threads, 0, st>>>(P);

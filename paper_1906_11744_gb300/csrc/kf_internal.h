@@ -179,7 +179,8 @@ struct FitParams {
   int* careful_list;      // [ns] positions (in order) of the tracks refitted with double-precision steps;
                           // the careful pass adds CAREFUL_DBL_BIT where the adjoint needs double steps
   unsigned* careful_count;  // zeroed before the launch
-  unsigned char* careful_flag;  // [ns] by track: 1 for the tracks of careful_list, else 0
+  unsigned char* careful_flag;  // [ns] by track: for the tracks of careful_list 1 + the step the FP32
+                                // pass stopped at (255 at most), else 0
   int* dbl_list;          // [ns] positions of the careful tracks with CAREFUL_DBL_BIT, packed
   unsigned* dbl_count;    // their number (zeroed before the careful pass)
   float* ckpt;            // [ckpt_slices][27][ns] by position: states before every ckpt_stride-th hit, or null
@@ -233,11 +234,13 @@ struct AdjParams {
 };
 
 // kf_adjoint.cu
-// Adjoint: zero the accumulators, the FP32 pass and the passes over the
-// fit's careful list (independent: either order or concurrently), then the
-// alignment gradient from its double-precision sums.
+// Adjoint: zero the accumulators, the FP32 pass, the passes over the fit's
+// careful list, without and with double-precision steps (independent: any
+// order or concurrently), then the alignment gradient from its
+// double-precision sums.
+enum { ADJ_MAIN = 0, ADJ_LIST = 1, ADJ_DBL = 2 };
 cudaError_t launch_adjoint_begin(const AdjParams& P, cudaStream_t st);
-cudaError_t launch_adjoint_pass(const AdjParams& P, bool careful, cudaStream_t st);
+cudaError_t launch_adjoint_pass(const AdjParams& P, int pass, cudaStream_t st);
 cudaError_t launch_adjoint_end(const AdjParams& P, cudaStream_t st);
 bool adjoint_stride_ok(int stride, int max_len);
 // kf_find.cu

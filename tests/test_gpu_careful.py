@@ -5,6 +5,8 @@ steps over the seed's hits then run in double); without it the listed ones are
 the loopers near their largest radius, taken on from where the FP32 passes
 stopped.  Tolerances are those of the parity tests.
 """
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -45,6 +47,38 @@ def test_careful_fit_list_sizes(n, loose):
     okc, ec = cov_close(fit["cov"].T[ok], C[ok], p[ok])
     assert okp.all(), ep
     assert okc.all(), ec
+
+
+def _loopers(n):
+    """The n tracks of lowest pT of many: most of them listed, many of them with double-precision steps."""
+    b = make_batch("c3", tracks=12 * n + 200)
+    sel = np.sort(np.argsort(-np.abs(b.params[3]))[:n])
+    return dataclasses.replace(b, params=np.ascontiguousarray(b.params[:, sel]), cov=np.ascontiguousarray(b.cov[:, sel]),
+                               seed_hits=np.ascontiguousarray(b.seed_hits[:, sel]), seed_sim=b.seed_sim[sel],
+                               seed_off=np.array([0, n], np.int32))
+
+
+@pytest.mark.parametrize("stride", [1, 4])
+@pytest.mark.parametrize("n", [1, 33, 153, 1500])
+def test_careful_adjoint_list_sizes(n, stride):
+    """Gradients of loopers, norm-wise within the 1e-3 of the adjoint's parity test."""
+    from paper_1906_11744_gb300 import KF_FIT_GIVEN
+    b = _loopers(n)
+    lists, nh = true_hit_lists(b, 0, b.det.n_layers)
+    lists, nh = lists[b.seed_sim], nh[b.seed_sim]
+    t = tracker_for(b, ckpt_stride=stride)
+    t.fit_tracks(KF_FIT_GIVEN, lists, nh)
+    g_align = np.zeros((b.det.n_layers, 2), np.float32)
+    g_hits = np.zeros((b.n_hits, 3), np.float32)
+    g_seed = np.zeros((6, n), np.float32)
+    t.fit_adjoint(g_align, g_hits, g_seed)
+    ok = t.get_fit()["status"] == 0
+    t.close()
+    assert ok.mean() >= 0.99
+    x, y, z, lay = b.event_hits(0)
+    _, ga, gh, gs, _ = oracle.fit_grad(b.det, b.params[:, ok], b.cov[:, ok], lists[ok], nh[ok], x, y, z, lay, b.align)
+    for g, ref in ((g_align, ga), (g_hits, gh), (g_seed[:, ok].T, gs)):
+        assert np.abs(g - ref).max() < 1e-3 * np.abs(ref).max()
 
 
 @pytest.mark.parametrize("cap", [0, 1])
