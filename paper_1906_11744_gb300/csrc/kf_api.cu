@@ -39,7 +39,7 @@ struct kf_ctx {
   // binning
   DevBuf hb, bin_cnt, bin_key, bin_rank, scan_tmp, bin_grouped, bin_gtab;
   // finding
-  DevBuf out_hits, out_n, out_chi2, out_p, out_C, keep, queue, counters, status, tangent, seed_order, check;
+  DevBuf out_hits, out_n, out_chi2, out_p, out_C, keep, queue, counters, status, tangent, seed_order;
   DevBuf sfit, sflag, skeys, x0map, rec;
   int rec_cap = 0;
   // duplicate removal scratch (the conflict lists also serve seed cleaning)
@@ -55,6 +55,7 @@ struct kf_ctx {
   int fit_source = KF_FIT_FOUND;
   FitParams last_fit;
   DevBuf adj_align_acc, adj_align, adj_hits, adj_seed;
+  int* bad = nullptr;  // two pinned host words the load kernels report bad input to
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   // What the captured graph baked in: the device address of every buffer and
@@ -119,48 +120,42 @@ void release(DevBuf& b) {
 
 cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
+// Event offsets to the device: as the load kernel's argument, or (many events)
+// by a copy of their own.
+cudaError_t offsets_arg(const std::vector<int>& h, void* dst, cudaStream_t st, OffsetArg* o) {
+  if (h.size() > (size_t)OFFSET_ARG)
+    return cudaMemcpyAsync(dst, h.data(), sizeof(int) * h.size(), cudaMemcpyHostToDevice, st);
+  o->n = (int)h.size();
+  std::copy(h.begin(), h.end(), o->v);
+  return cudaSuccess;
+}
+
+// The copies of c that come from host memory are made here and leave the list
+// (a load kernel makes those from device memory).
+cudaError_t from_host(CopyList* c, int device_ptrs, cudaStream_t st) {
+  if (device_ptrs) return cudaSuccess;
+  for (int k = 0; k < c->n; ++k) {
+    const cudaError_t e = cudaMemcpyAsync(c->dst[k], c->src[k], c->bytes[k], cudaMemcpyHostToDevice, st);
+    if (e != cudaSuccess) return e;
+  }
+  c->n = 0;
+  return cudaSuccess;
+}
+
+// Results out: to device memory in one launch, to host memory by copies.
+cudaError_t get_all(const CopyList& c, int device_ptrs, int num_sms, cudaStream_t st) {
+  if (device_ptrs) return launch_copy(c, num_sms, st);
+  for (int k = 0; k < c.n; ++k) {
+    const cudaError_t e = cudaMemcpyAsync(c.dst[k], c.src[k], c.bytes[k], cudaMemcpyDeviceToHost, st);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 // Copy n bytes into a device buffer from a host or device source.
 cudaError_t put(void* dst, const void* src, size_t n, int device_ptrs, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
   return cudaMemcpyAsync(dst, src, n, device_ptrs ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st);
-}
-
-cudaError_t get(void* dst, const void* src, size_t n, int device_ptrs, cudaStream_t st) {
-  if (n == 0) return cudaSuccess;
-  return cudaMemcpyAsync(dst, src, n, device_ptrs ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st);
-}
-
-// Input checks on the device (after the copies; works for host and device
-// arrays alike): any value outside [0, hi) sets *bad.
-__global__ void k_check_range(const int* v, int n, int hi, int* bad) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    if (v[i] < 0 || v[i] >= hi) *bad = 1;
-}
-// Seed hit indices (three per seed, [3][n]) against their event's hit count;
-// the hits must lie on barrel layers (*bad = 2 otherwise).
-__global__ void k_check_seed_hits(const int* sh, const int* seed_event, const int* hit_off, const int* hlayer,
-                                  int n_layers, int n, int* bad) {
-  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
-    const int e = seed_event[s];
-    const int nh = hit_off[e + 1] - hit_off[e];
-    for (int k = 0; k < 3; ++k) {
-      const int h = sh[(size_t)k * n + s];
-      if (h < 0 || h >= nh) *bad = 1;
-      else if (hlayer[hit_off[e] + h] >= n_layers) atomicMax(bad, 2);
-    }
-  }
-}
-
-// Event of every seed from the seed offsets (binary search).
-__global__ void k_seed_event(const int* seed_off, int n_events, int n, int* out) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= n) return;
-  int lo = 0, hi = n_events - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (seed_off[mid] <= s) lo = mid; else hi = mid - 1;
-  }
-  out[s] = lo;
 }
 
 __global__ void k_align(const float* off, const DevGeom g, Align4* out) {
@@ -342,6 +337,7 @@ int kf_create(const kf_detector* det, const kf_config* cfg, kf_ctx** out) {
     if (e == cudaSuccess) e = cudaMemcpy(ctx->eta_lut.p, lut.data(), lut.size(), cudaMemcpyHostToDevice);
   }
   if (e == cudaSuccess) e = grow(ctx->queue, 64);
+  if (e == cudaSuccess) e = cudaHostAlloc(&ctx->bad, 2 * sizeof(int), cudaHostAllocMapped);
   if (e == cudaSuccess) {
     int least = 0, greatest = 0;
     e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
@@ -372,7 +368,7 @@ static std::vector<DevBuf*> all_bufs(kf_ctx* ctx) {
   return {&ctx->hx, &ctx->hy, &ctx->hz, &ctx->hlayer, &ctx->hit_off, &ctx->seed_off, &ctx->sp,
                     &ctx->sc, &ctx->sh, &ctx->seed_event, &ctx->align_raw, &ctx->align4, &ctx->eta_edges, &ctx->eta_lut, &ctx->hb,
                     &ctx->bin_cnt, &ctx->bin_key, &ctx->bin_rank, &ctx->scan_tmp, &ctx->bin_grouped, &ctx->bin_gtab, &ctx->out_hits,
-                    &ctx->out_n, &ctx->out_chi2, &ctx->out_p, &ctx->out_C, &ctx->keep, &ctx->queue, &ctx->tangent, &ctx->seed_order, &ctx->check,
+                    &ctx->out_n, &ctx->out_chi2, &ctx->out_p, &ctx->out_C, &ctx->keep, &ctx->queue, &ctx->tangent, &ctx->seed_order,
                     &ctx->counters, &ctx->status, &ctx->dd_head, &ctx->dd_next, &ctx->dd_conf,
                     &ctx->dd_nconf, &ctx->dd_state, &ctx->given_lists, &ctx->given_n, &ctx->fit_p,
                     &ctx->fit_C, &ctx->fit_chi2, &ctx->fit_status, &ctx->careful_list,
@@ -393,6 +389,7 @@ int kf_destroy(kf_ctx* ctx) {
   if (ctx->exec) cudaGraphExecDestroy(ctx->exec);
   if (ctx->graph) cudaGraphDestroy(ctx->graph);
   for (DevBuf* b : all_bufs(ctx)) release(*b);
+  if (ctx->bad) cudaFreeHost(ctx->bad);
   delete ctx;
   return KF_OK;
 }
@@ -426,30 +423,26 @@ int kf_load_hits(kf_ctx* ctx, int n_events, const int* ev_offsets, const float* 
   CK(grow(ctx->bin_grouped, sizeof(float4) * n));
   CK(grow(ctx->bin_gtab, sizeof(unsigned) * bin_group_elems(n_events, ctx->g.n_surf, ctx->g.n_eta, ctx->g.n_phi)));
   CK(grow(ctx->dd_head, sizeof(unsigned) * ((size_t)n + n_events)));
-  CK(put(ctx->hx.p, x, sizeof(float) * n, device_ptrs, st));
-  CK(put(ctx->hy.p, y, sizeof(float) * n, device_ptrs, st));
-  CK(put(ctx->hz.p, z, sizeof(float) * n, device_ptrs, st));
-  CK(put(ctx->hlayer.p, layer, sizeof(int) * n, device_ptrs, st));
   ctx->hit_off_h.assign(ev_offsets, ev_offsets + n_events + 1);
-  CK(cudaMemcpyAsync(ctx->hit_off.p, ctx->hit_off_h.data(), sizeof(int) * (n_events + 1),
-                     cudaMemcpyHostToDevice, st));
+  CopyList c;
+  c.add(ctx->hx.p, x, sizeof(float) * n);
+  c.add(ctx->hy.p, y, sizeof(float) * n);
+  c.add(ctx->hz.p, z, sizeof(float) * n);
+  c.add(ctx->hlayer.p, layer, sizeof(int) * n);
+  CK(from_host(&c, device_ptrs, st));
+  OffsetArg off;
+  CK(offsets_arg(ctx->hit_off_h, ctx->hit_off.p, st, &off));
   ctx->found = ctx->deduped = ctx->fitted = false;
   // Seed hit indices were checked against the previous hit offsets: the seeds
   // must be loaded again before finding, fitting or tuning.
   ctx->n_seed_events = -1;
   // Layer indices checked on the device (the caller's buffers are in use until
   // the synchronization below).
-  int bad = 0;
-  CK(grow(ctx->check, 64));
-  CK(cudaMemsetAsync(ctx->check.p, 0, sizeof(int), st));
-  if (n > 0) {
-    k_check_range<<<std::min((n + 255) / 256, 4 * ctx->num_sms), 256, 0, st>>>(ptr<int>(ctx->hlayer), n,
-                                                                               ctx->g.n_surf, ptr<int>(ctx->check));
-    CK(cudaGetLastError());
-  }
-  CK(cudaMemcpyAsync(&bad, ctx->check.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+  ctx->bad[0] = 0;
+  CK(launch_load_hits(c, device_ptrs ? layer : ptr<int>(ctx->hlayer), n, ctx->g.n_surf, off, ptr<int>(ctx->hit_off),
+                      ctx->bad, ctx->num_sms, st));
   CK(cudaStreamSynchronize(st));
-  if (bad) {
+  if (ctx->bad[0]) {
     ctx->n_events = 0;
     ctx->n_hits = -1;
     return fail(ctx, KF_ERR_ARG, "kf_load_hits: layer index out of range");
@@ -516,32 +509,25 @@ int kf_load_seeds(kf_ctx* ctx, int n_events, const int* ev_offsets, const float*
     CK(grow(ctx->sc_list, sizeof(int) * (size_t)n));
     CK(grow(ctx->sc_list_cnt, sizeof(int) * (size_t)n_events));
   }
-  CK(put(ctx->sp.p, params, sizeof(float) * 6 * (size_t)n, device_ptrs, st));
-  CK(put(ctx->sc.p, cov, sizeof(float) * 21 * (size_t)n, device_ptrs, st));
-  CK(put(ctx->sh.p, seed_hits, sizeof(int) * 3 * (size_t)n, device_ptrs, st));
   ctx->seed_off_h.assign(ev_offsets, ev_offsets + n_events + 1);
-  CK(cudaMemcpyAsync(ctx->seed_off.p, ctx->seed_off_h.data(), sizeof(int) * (n_events + 1),
-                     cudaMemcpyHostToDevice, st));
-  if (n > 0) {
-    k_seed_event<<<(n + 255) / 256, 256, 0, st>>>(ptr<int>(ctx->seed_off), n_events, n, ptr<int>(ctx->seed_event));
-    CK(cudaGetLastError());
-    CK(launch_seed_order(ptr<float>(ctx->sp) + 5 * (size_t)n, ptr<int>(ctx->seed_off), n_events,
-                         ptr<int>(ctx->seed_order), st));
-  }
-  CK(cudaMemsetAsync(ctx->keep.p, 1, (size_t)n, st));
+  CopyList c;
+  c.add(ctx->sp.p, params, sizeof(float) * 6 * (size_t)n);
+  c.add(ctx->sc.p, cov, sizeof(float) * 21 * (size_t)n);
+  c.add(ctx->sh.p, seed_hits, sizeof(int) * 3 * (size_t)n);
+  CK(from_host(&c, device_ptrs, st));
+  OffsetArg off;
+  CK(offsets_arg(ctx->seed_off_h, ctx->seed_off.p, st, &off));
   ctx->found = ctx->deduped = ctx->fitted = false;
   // Seed hit indices checked on the device against their event's hits.
-  int bad = 0;
-  CK(grow(ctx->check, 64));
-  CK(cudaMemsetAsync(ctx->check.p, 0, sizeof(int), st));
-  if (n > 0) {
-    k_check_seed_hits<<<std::min((n + 255) / 256, 4 * ctx->num_sms), 256, 0, st>>>(
-        ptr<int>(ctx->sh), ptr<int>(ctx->seed_event), ptr<int>(ctx->hit_off), ptr<int>(ctx->hlayer),
-        ctx->g.n_layers, n, ptr<int>(ctx->check));
-    CK(cudaGetLastError());
-  }
-  CK(cudaMemcpyAsync(&bad, ctx->check.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+  ctx->bad[0] = ctx->bad[1] = 0;
+  CK(launch_load_seeds(c, device_ptrs ? seed_hits : ptr<int>(ctx->sh), n, n_events, off, ptr<int>(ctx->seed_off),
+                       ptr<int>(ctx->hit_off), ptr<int>(ctx->hlayer), ctx->g.n_layers, ptr<int>(ctx->seed_event),
+                       ptr<unsigned char>(ctx->keep), ctx->bad, ctx->num_sms, st));
+  if (n > 0)
+    CK(launch_seed_order(ptr<float>(ctx->sp) + 5 * (size_t)n, ptr<int>(ctx->seed_off), n_events,
+                         ptr<int>(ctx->seed_order), st));
   CK(cudaStreamSynchronize(st));
+  const int bad = ctx->bad[0] ? 1 : ctx->bad[1] ? 2 : 0;
   if (bad) {
     ctx->n_seed_events = -1;
     return fail(ctx, KF_ERR_ARG, bad == 1 ? "kf_load_seeds: seed hit index out of range"
@@ -585,8 +571,8 @@ int kf_set_alignment(kf_ctx* ctx, const float* offsets, int device_ptrs, void* s
   cudaStream_t st = S(stream);
   const int L = ctx->g.n_layers;
   CK(grow(ctx->align_raw, sizeof(float) * 2 * KF_MAX_LAYERS));
-  if (offsets) CK(put(ctx->align_raw.p, offsets, sizeof(float) * 2 * L, device_ptrs, st));
-  k_align<<<1, KF_MAX_LAYERS, 0, st>>>(offsets ? ptr<float>(ctx->align_raw) : nullptr, ctx->g,
+  if (offsets && !device_ptrs) CK(put(ctx->align_raw.p, offsets, sizeof(float) * 2 * L, 0, st));
+  k_align<<<1, KF_MAX_LAYERS, 0, st>>>(offsets && !device_ptrs ? ptr<float>(ctx->align_raw) : offsets, ctx->g,
                                        ptr<Align4>(ctx->align4));
   CK(cudaGetLastError());
   if (!device_ptrs) CK(cudaStreamSynchronize(st));
@@ -731,16 +717,21 @@ int kf_find_tracks(kf_ctx* ctx, void* stream) {
     return fail(ctx, KF_ERR_STATE, "kf_find_tracks: load hits and seeds first");
   cudaStream_t st = S(stream);
   const size_t cells = (size_t)ctx->g.n_surf * ctx->g.n_eta * ctx->g.n_phi;
-  CK(cudaMemsetAsync(ctx->counters.p, 0, 8 * KF_N_COUNTERS, st));
-  CK(cudaMemsetAsync(ctx->keep.p, 1, (size_t)ctx->n_seeds, st));
   auto find_main = [&](const FindParams& P) {
     const bool cap = ctx->regcap || (ctx->auto_cap && (long long)(P.s_end - P.s_begin) * ctx->g.max_cands > AUTO_CAP_CANDS);
     const int bps = cap && !ctx->regcap ? ctx->cap_blocks_per_sm : ctx->blocks_per_sm;
     return launch_find_main(P, ctx->lanes, cap, ctx->threads, ctx->num_sms * bps, st);
   };
+  auto begin = [&](size_t n_table) {
+    return launch_find_begin(FindBegin{ptr<unsigned long long>(ctx->counters), ptr<unsigned>(ctx->queue),
+                                       ptr<unsigned>(ctx->bin_gtab), ptr<unsigned char>(ctx->keep), KF_N_COUNTERS, 16,
+                                       n_table, ctx->n_seeds},
+                             ctx->num_sms, st);
+  };
   if (!ctx->per_event) {
     BinParams B = bin_params(ctx);
     stage_mark(ctx, 0, st);
+    CK(begin(bin_table_elems(B, ctx->n_events)));
     CK(launch_bin(B, 0, ctx->n_bins_total, 0u, ctx->max_event_hits, ptr<unsigned>(ctx->scan_tmp),
                   ctx->scan_tmp.bytes / sizeof(unsigned), st));
     stage_mark(ctx, 1, st);
@@ -752,14 +743,15 @@ int kf_find_tracks(kf_ctx* ctx, void* stream) {
       P.order = ptr<int>(ctx->clean_order);
       P.kept_cnt = ptr<int>(ctx->kept_cnt);
     }
-    CK(cudaMemsetAsync(ctx->queue.p, 0, 64, st));
     stage_mark(ctx, 2, st);
     CK(find_main(P));
     CK(launch_find_careful(P, ctx->lanes, careful_grid(ctx, P.s_end - P.s_begin), st));
     stage_mark(ctx, 3, st);
   } else {
+    CK(begin(0));
     for (int e = 0; e < ctx->n_events; ++e) {
       BinParams B = bin_params(ctx);
+      CK(cudaMemsetAsync(ctx->bin_gtab.p, 0, sizeof(unsigned) * bin_table_elems(B, 1), st));
       B.h_begin = ctx->hit_off_h[e];
       B.h_end = ctx->hit_off_h[e + 1];
       CK(launch_bin(B, (size_t)e * cells, cells, (unsigned)ctx->hit_off_h[e],
@@ -1007,12 +999,14 @@ int kf_get_tracks(kf_ctx* ctx, int* hits, int* n_found, float* chi2, float* para
   if (!ctx->found) return fail(ctx, KF_ERR_STATE, "kf_get_tracks: run kf_find_tracks first");
   cudaStream_t st = S(stream);
   const size_t n = (size_t)ctx->n_seeds, L = (size_t)ctx->g.n_surf;
-  if (hits) CK(get(hits, ctx->out_hits.p, sizeof(int) * n * L, device_ptrs, st));
-  if (n_found) CK(get(n_found, ctx->out_n.p, sizeof(int) * n, device_ptrs, st));
-  if (chi2) CK(get(chi2, ctx->out_chi2.p, sizeof(float) * n, device_ptrs, st));
-  if (params) CK(get(params, ctx->out_p.p, sizeof(float) * 6 * n, device_ptrs, st));
-  if (cov) CK(get(cov, ctx->out_C.p, sizeof(float) * 21 * n, device_ptrs, st));
-  if (keep) CK(get(keep, ctx->keep.p, n, device_ptrs, st));
+  CopyList c;
+  c.add(hits, ctx->out_hits.p, sizeof(int) * n * L);
+  c.add(n_found, ctx->out_n.p, sizeof(int) * n);
+  c.add(chi2, ctx->out_chi2.p, sizeof(float) * n);
+  c.add(params, ctx->out_p.p, sizeof(float) * 6 * n);
+  c.add(cov, ctx->out_C.p, sizeof(float) * 21 * n);
+  c.add(keep, ctx->keep.p, n);
+  CK(get_all(c, device_ptrs, ctx->num_sms, st));
   if (!device_ptrs) return check_status(ctx, st);
   return KF_OK;
 }
@@ -1022,10 +1016,12 @@ int kf_get_fit(kf_ctx* ctx, float* params, float* cov, float* chi2, int* status,
   if (!ctx->fitted) return fail(ctx, KF_ERR_STATE, "kf_get_fit: run kf_fit_tracks first");
   cudaStream_t st = S(stream);
   const size_t n = (size_t)ctx->n_seeds;
-  if (params) CK(get(params, ctx->fit_p.p, sizeof(float) * 6 * n, device_ptrs, st));
-  if (cov) CK(get(cov, ctx->fit_C.p, sizeof(float) * 21 * n, device_ptrs, st));
-  if (chi2) CK(get(chi2, ctx->fit_chi2.p, sizeof(float) * n, device_ptrs, st));
-  if (status) CK(get(status, ctx->fit_status.p, sizeof(int) * n, device_ptrs, st));
+  CopyList c;
+  c.add(params, ctx->fit_p.p, sizeof(float) * 6 * n);
+  c.add(cov, ctx->fit_C.p, sizeof(float) * 21 * n);
+  c.add(chi2, ctx->fit_chi2.p, sizeof(float) * n);
+  c.add(status, ctx->fit_status.p, sizeof(int) * n);
+  CK(get_all(c, device_ptrs, ctx->num_sms, st));
   if (!device_ptrs) return check_status(ctx, st);
   return KF_OK;
 }
@@ -1146,17 +1142,15 @@ int kf_get_gradient(kf_ctx* ctx, float* g_align, float* g_hits, float* g_seed, i
   if (!ctx) return KF_ERR_ARG;
   if (!ctx->adj_align.p) return fail(ctx, KF_ERR_STATE, "kf_get_gradient: no gradient computed");
   cudaStream_t st = S(stream);
-  if (g_align) CK(get(g_align, ctx->adj_align.p, sizeof(float) * 2 * ctx->g.n_layers, device_ptrs, st));
-  if (g_hits) {
-    if (ctx->adj_hits.bytes < sizeof(float) * 3 * (size_t)ctx->n_hits)
-      return fail(ctx, KF_ERR_STATE, "kf_get_gradient: no hit gradient kept");
-    CK(get(g_hits, ctx->adj_hits.p, sizeof(float) * 3 * (size_t)ctx->n_hits, device_ptrs, st));
-  }
-  if (g_seed) {
-    if (ctx->adj_seed.bytes < sizeof(float) * 6 * (size_t)ctx->n_seeds)
-      return fail(ctx, KF_ERR_STATE, "kf_get_gradient: no seed gradient kept");
-    CK(get(g_seed, ctx->adj_seed.p, sizeof(float) * 6 * (size_t)ctx->n_seeds, device_ptrs, st));
-  }
+  if (g_hits && ctx->adj_hits.bytes < sizeof(float) * 3 * (size_t)ctx->n_hits)
+    return fail(ctx, KF_ERR_STATE, "kf_get_gradient: no hit gradient kept");
+  if (g_seed && ctx->adj_seed.bytes < sizeof(float) * 6 * (size_t)ctx->n_seeds)
+    return fail(ctx, KF_ERR_STATE, "kf_get_gradient: no seed gradient kept");
+  CopyList c;
+  c.add(g_align, ctx->adj_align.p, sizeof(float) * 2 * ctx->g.n_layers);
+  c.add(g_hits, ctx->adj_hits.p, sizeof(float) * 3 * (size_t)ctx->n_hits);
+  c.add(g_seed, ctx->adj_seed.p, sizeof(float) * 6 * (size_t)ctx->n_seeds);
+  CK(get_all(c, device_ptrs, ctx->num_sms, st));
   if (!device_ptrs) return check_status(ctx, st);
   return KF_OK;
 }

@@ -360,10 +360,17 @@ size_t bin_group_elems(int n_events, int n_layers, int n_eta, int n_phi) {
   return 3 * ((size_t)n_events * n_layers * chunks_of(n_eta, n_phi).n + 1);
 }
 
+size_t bin_table_elems(const BinParams& P, int n_events) {
+  return P.g.n_phi <= CHUNK_CELLS && P.grouped && P.gtab
+             ? (size_t)n_events * P.g.n_surf * chunks_of(P.g.n_eta, P.g.n_phi).n
+             : 0;
+}
+
 // Bins the hits [P.h_begin, P.h_end), which must be whole events whose cells
 // are cnt[bin_begin, bin_begin + n_bins); `first_pos` is the binned position
 // of the first of them (the number of hits of all earlier events).
-// max_event_hits: the largest hit count of those events.
+// max_event_hits: the largest hit count of those events.  The first
+// bin_table_elems() bucket counts are zero.
 cudaError_t launch_bin(const BinParams& P, size_t bin_begin, size_t n_bins, unsigned first_pos, int max_event_hits,
                        unsigned* scan_tmp, size_t scan_tmp_elems_, cudaStream_t st) {
   const int n_hits = P.h_end - P.h_begin;
@@ -374,8 +381,6 @@ cudaError_t launch_bin(const BinParams& P, size_t bin_begin, size_t n_bins, unsi
     const int n_ev = (int)(n_bins / per_event);
     const int nb_ev = P.g.n_surf * ch.n;
     const int nb = n_ev * nb_ev;  // buckets of the launch
-    cudaError_t err = cudaMemsetAsync(P.gtab, 0, sizeof(unsigned) * (size_t)nb, st);
-    if (err != cudaSuccess) return err;
     const dim3 ggrid((max_event_hits + GROUP_HITS - 1) / GROUP_HITS, n_ev);
     if (n_hits > 0 && ggrid.x > 0) k_group<true><<<ggrid, GROUP_THREADS, sizeof(unsigned) * nb_ev, st>>>(P, e_first, nb);
     k_group_scan<<<1, SCAN_THREADS, 0, st>>>(P, nb, first_pos, bin_begin + n_bins);

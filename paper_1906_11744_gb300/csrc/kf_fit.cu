@@ -97,12 +97,14 @@ __device__ __forceinline__ int order_key(const FitParams& P, int t) {
   return min(max(P.n_list[t], 0), ORDER_BINS - 1);
 }
 
-// One block per window: counts per hit count, an exclusive prefix over the
+// One block per window (the first one also empties the careful pass's lists):
+// counts per hit count, an exclusive prefix over the
 // counts from the longest down, then each track's position (one shared-memory
 // atomic per hit count and warp).
 __global__ void __launch_bounds__(ORDER_THREADS) k_fit_order(const FitParams P) {
   static_assert(ORDER_BINS == 64, "two bins per lane");
   __shared__ unsigned cnt[ORDER_BINS], cur[ORDER_BINS];
+  if (blockIdx.x == 0 && threadIdx.x == 0) *P.careful_count = *P.dbl_count = 0u;
   const int w0 = blockIdx.x * ORDER_WINDOW;
   const int w1 = min(P.ns, w0 + ORDER_WINDOW);
   for (int b = threadIdx.x; b < ORDER_BINS; b += blockDim.x) cnt[b] = 0u;
@@ -318,8 +320,6 @@ cudaError_t launch_fit_unkept(const FitParams& P, cudaStream_t st) {
 
 cudaError_t launch_fit_main(const FitParams& P, cudaStream_t st) {
   if (P.ns <= 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(P.careful_count, 0, sizeof(unsigned), st);
-  if (e != cudaSuccess) return e;
   k_fit_order<<<(P.ns + ORDER_WINDOW - 1) / ORDER_WINDOW, ORDER_THREADS, 0, st>>>(P);
   const int blocks = (P.ns + FIT_THREADS - 1) / FIT_THREADS;
   if (P.g.n_disks > 0) k_fit<true><<<blocks, FIT_THREADS, 0, st>>>(P);
@@ -334,8 +334,6 @@ cudaError_t launch_fit_careful(const FitParams& P, cudaStream_t st) {
   // striding over however many there are
   const int threads = 32;
   const int careful_blocks = std::max(P.ns / (64 * threads) + 1, std::min(P.ns, CAREFUL_BLOCKS));
-  cudaError_t e = cudaMemsetAsync(P.dbl_count, 0, sizeof(unsigned), st);
-  if (e != cudaSuccess) return e;
   if (P.g.n_disks > 0) k_fit_careful<true><<<careful_blocks, threads, 0, st>>>(P);
   else k_fit_careful<false><<<careful_blocks, threads, 0, st>>>(P);
   return cudaGetLastError();

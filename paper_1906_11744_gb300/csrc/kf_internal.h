@@ -178,11 +178,11 @@ struct FitParams {
   int* fit_status;        // [ns]
   int* careful_list;      // [ns] positions (in order) of the tracks refitted with double-precision steps;
                           // the careful pass adds CAREFUL_DBL_BIT where the adjoint needs double steps
-  unsigned* careful_count;  // zeroed before the launch
+  unsigned* careful_count;  // zeroed by launch_fit_main
   unsigned char* careful_flag;  // [ns] by track: for the tracks of careful_list 1 + the step the FP32
                                 // pass stopped at (255 at most), else 0
   int* dbl_list;          // [ns] positions of the careful tracks with CAREFUL_DBL_BIT, packed
-  unsigned* dbl_count;    // their number (zeroed before the careful pass)
+  unsigned* dbl_count;    // their number (zeroed by launch_fit_main)
   float* ckpt;            // [ckpt_slices][27][ns] by position: states before every ckpt_stride-th hit, or null
   int ckpt_stride;
   int ckpt_slices;        // checkpoints per track the buffer holds
@@ -233,6 +233,47 @@ struct AdjParams {
   const int* order;            // the fit's track order (position -> track)
 };
 
+// kf_copy.cu
+// Up to six copies of one launch.
+struct CopyList {
+  int n = 0;
+  void* dst[6];
+  const void* src[6];
+  size_t bytes[6];
+  void add(void* d, const void* s, size_t b) {
+    if (!d || b == 0) return;
+    dst[n] = d;
+    src[n] = s;
+    bytes[n++] = b;
+  }
+};
+// Event offsets as a kernel argument (n = 0: they are copied instead).
+constexpr int OFFSET_ARG = 128;
+struct OffsetArg {
+  int n = 0;
+  int v[OFFSET_ARG];
+};
+// What a finding call starts from: counters and queue zero, keep flags set, and
+// (batched form) the binning's bucket counts zero.
+struct FindBegin {
+  unsigned long long* counters;
+  unsigned* queue;
+  unsigned* table;
+  unsigned char* keep;
+  int n_counters, n_queue;
+  size_t n_table;
+  int n_keep;
+};
+cudaError_t launch_copy(const CopyList& c, int num_sms, cudaStream_t st);
+// Copies, offsets and checks of kf_load_hits / kf_load_seeds; layer, sh: where
+// the checked values are (the source or the copy); bad[2]: host memory, zeroed
+// by the caller, read after a synchronization.
+cudaError_t launch_load_hits(const CopyList& c, const int* layer, int n, int n_surf, const OffsetArg& o, int* hit_off,
+                             int* bad, int num_sms, cudaStream_t st);
+cudaError_t launch_load_seeds(const CopyList& c, const int* sh, int n, int n_events, const OffsetArg& o, int* seed_off,
+                              const int* hit_off, const int* hlayer, int n_layers, int* seed_event,
+                              unsigned char* keep, int* bad, int num_sms, cudaStream_t st);
+cudaError_t launch_find_begin(const FindBegin& b, int num_sms, cudaStream_t st);
 // kf_adjoint.cu
 // Adjoint: zero the accumulators, the FP32 pass, the passes over the fit's
 // careful list, without and with double-precision steps (independent: any
@@ -267,6 +308,9 @@ cudaError_t launch_find_careful_disk(const FindParams& P, int lanes, int grid, c
 // kf_bin.cu
 cudaError_t launch_bin(const BinParams& P, size_t bin_begin, size_t n_bins, unsigned first_pos, int max_event_hits,
                        unsigned* scan_tmp, size_t scan_tmp_elems, cudaStream_t st);
+// Bucket counts (BinParams::gtab) that launch_bin expects zeroed; 0: none (the
+// general form).
+size_t bin_table_elems(const BinParams& P, int n_events);
 size_t scan_tmp_elems(size_t n);
 size_t bin_group_elems(int n_events, int n_layers, int n_eta, int n_phi);
 // kf_dedup.cu
