@@ -163,7 +163,15 @@ constexpr int CELL_THREADS = 256;
 constexpr int CELL_WORDS = CHUNK_CELLS / 2;                    // two 16-bit counters per word
 constexpr int CELL_SMEM_WORDS = CELL_WORDS + CELL_WORDS / 32;  // one pad word per 32
 constexpr int GROUP_THREADS = 256;
-constexpr int GROUP_HITS = 4096;  // hits of one event per grouping block
+// Hits of one event per grouping block: at most GROUP_HITS (a block's flush of
+// its bucket counts costs as much as some thousand hits), fewer where that
+// would leave SMs idle: 256 per block for one 2,500-track event, whose two
+// grouping passes took 20 and 36 us in 11 blocks.
+constexpr int GROUP_HITS = 4096, GROUP_BLOCKS = 304;
+inline int group_hits(int n_hits) {
+  const int per = (n_hits / GROUP_BLOCKS + GROUP_THREADS - 1) / GROUP_THREADS * GROUP_THREADS;
+  return per < GROUP_THREADS ? GROUP_THREADS : per > GROUP_HITS ? GROUP_HITS : per;
+}
 __device__ __forceinline__ int pad_word(int w) { return w + (w >> 5); }
 
 struct Chunks {
@@ -184,19 +192,19 @@ __device__ __forceinline__ int bucket_in_event(const BinParams& P, int i, Chunks
   return l * ch.n + row_of(P, l, P.hx[i], P.hy[i], P.hz[i]) / ch.rows;
 }
 
-// Grid (ceil(max event hits / GROUP_HITS), events of the launch): block (c, e)
-// takes hits [GROUP_HITS c, GROUP_HITS (c + 1)) of event e_first + e.
+// Grid (ceil(max event hits / per), events of the launch): block (c, e) takes
+// hits [per c, per (c + 1)) of event e_first + e.
 // COUNT: per-block histogram of the event's buckets added to the global
 // counts.  SCATTER: per-block bases from the global cursors, hits written to
 // the grouped array at base + rank within the block.
 template <bool COUNT>
-__global__ void __launch_bounds__(GROUP_THREADS) k_group(const BinParams P, int e_first, int n_buckets) {
+__global__ void __launch_bounds__(GROUP_THREADS) k_group(const BinParams P, int e_first, int n_buckets, int per) {
   extern __shared__ unsigned hist[];  // buckets of one event
   const Chunks ch = chunks_of(P.g.n_eta, P.g.n_phi);
   const int nb_ev = P.g.n_surf * ch.n;
   const int ev = e_first + blockIdx.y;
-  const int h0 = P.hit_off[ev] + blockIdx.x * GROUP_HITS;
-  const int h1 = min(P.hit_off[ev + 1], h0 + GROUP_HITS);
+  const int h0 = P.hit_off[ev] + blockIdx.x * per;
+  const int h1 = min(P.hit_off[ev + 1], h0 + per);
   if (h0 >= h1) return;
   for (int k = threadIdx.x; k < nb_ev; k += blockDim.x) hist[k] = 0u;
   __syncthreads();
@@ -381,11 +389,12 @@ cudaError_t launch_bin(const BinParams& P, size_t bin_begin, size_t n_bins, unsi
     const int n_ev = (int)(n_bins / per_event);
     const int nb_ev = P.g.n_surf * ch.n;
     const int nb = n_ev * nb_ev;  // buckets of the launch
-    const dim3 ggrid((max_event_hits + GROUP_HITS - 1) / GROUP_HITS, n_ev);
-    if (n_hits > 0 && ggrid.x > 0) k_group<true><<<ggrid, GROUP_THREADS, sizeof(unsigned) * nb_ev, st>>>(P, e_first, nb);
+    const int per = group_hits(n_hits);
+    const dim3 ggrid((max_event_hits + per - 1) / per, n_ev);
+    if (n_hits > 0 && ggrid.x > 0) k_group<true><<<ggrid, GROUP_THREADS, sizeof(unsigned) * nb_ev, st>>>(P, e_first, nb, per);
     k_group_scan<<<1, SCAN_THREADS, 0, st>>>(P, nb, first_pos, bin_begin + n_bins);
     if (n_hits > 0 && ggrid.x > 0)
-      k_group<false><<<ggrid, GROUP_THREADS, 2 * sizeof(unsigned) * nb_ev, st>>>(P, e_first, nb);
+      k_group<false><<<ggrid, GROUP_THREADS, 2 * sizeof(unsigned) * nb_ev, st>>>(P, e_first, nb, per);
     const size_t smem = sizeof(unsigned) * CELL_SMEM_WORDS;
     if (nb > 0) k_cells<<<nb, CELL_THREADS, smem, st>>>(P, e_first, nb);
     return cudaGetLastError();
