@@ -184,12 +184,9 @@ class Tracker:
 
     @staticmethod
     def _alloc(device, **specs):
-        out = {}
-        for name, (shape, dt) in specs.items():
-            if device is None:
-                out[name] = np.zeros(shape, dtype=np.dtype(dt))
-            else:
-                import torch
-                tdt = {"i4": torch.int32, "f4": torch.float32, "u1": torch.uint8}[dt]
-                out[name] = torch.zeros(shape, dtype=tdt, device=device)
-        return out
+        """Output arrays, uninitialized (the library writes every element)."""
+        if device is None:
+            return {name: np.empty(shape, dtype=dt) for name, (shape, dt) in specs.items()}
+        import torch
+        tdt = {"i4": torch.int32, "f4": torch.float32, "u1": torch.uint8}
+        return {name: torch.empty(shape, dtype=tdt[dt], device=device) for name, (shape, dt) in specs.items()}

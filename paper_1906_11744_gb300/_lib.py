@@ -127,20 +127,24 @@ def _is_torch(a):
     return type(a).__module__.startswith("torch")
 
 
+_TORCH_DTYPE = None  # numpy type -> torch dtype, once torch is in use
+
+
 def _arg(a, dtype):
     """(pointer, keepalive, device flag) for a torch tensor or array-like."""
+    global _TORCH_DTYPE
     if a is None:
         return None, None, None
     if _is_torch(a):
-        import torch
-        tdt = {np.float32: torch.float32, np.int32: torch.int32, np.uint8: torch.uint8}[dtype]
+        if _TORCH_DTYPE is None:
+            import torch
+            _TORCH_DTYPE = {np.float32: torch.float32, np.int32: torch.int32, np.uint8: torch.uint8}
+        tdt = _TORCH_DTYPE[dtype]
         if a.dtype != tdt or not a.is_contiguous():
             a = a.to(tdt).contiguous()
-        if a.is_cuda:
-            return ctypes.c_void_p(a.data_ptr()), a, 1
-        return ctypes.c_void_p(a.data_ptr()), a, 0
+        return a.data_ptr(), a, 1 if a.is_cuda else 0
     arr = np.ascontiguousarray(a, dtype=dtype)
-    return arr.ctypes.data_as(ctypes.c_void_p), arr, 0
+    return arr.ctypes.data, arr, 0
 
 
 def _stream(stream):
@@ -176,7 +180,7 @@ def kf_load_hits(ctx, ev_offsets, x, y, z, layer, stream=None):
     py, ky, fy = _arg(y, np.float32)
     pz, kz, fz = _arg(z, np.float32)
     pl, kl, fl = _arg(layer, np.int32)
-    rc = load().kf_load_hits(ctx, off.size - 1, off.ctypes.data_as(_P), px, py, pz, pl,
+    rc = load().kf_load_hits(ctx, off.size - 1, off.ctypes.data, px, py, pz, pl,
                              _flag(fx, fy, fz, fl), _stream(stream))
     _check(ctx, rc, "kf_load_hits")
 
@@ -186,7 +190,7 @@ def kf_load_seeds(ctx, ev_offsets, params, cov, seed_hits, stream=None):
     pp, kp, fp = _arg(params, np.float32)
     pc, kc, fc = _arg(cov, np.float32)
     ps, ks, fs = _arg(seed_hits, np.int32)
-    rc = load().kf_load_seeds(ctx, off.size - 1, off.ctypes.data_as(_P), pp, pc, ps, _flag(fp, fc, fs),
+    rc = load().kf_load_seeds(ctx, off.size - 1, off.ctypes.data, pp, pc, ps, _flag(fp, fc, fs),
                               _stream(stream))
     _check(ctx, rc, "kf_load_seeds")
 
@@ -261,7 +265,7 @@ def kf_launch_graph(ctx, stream=None):
 def kf_autotune(ctx, stream=None, max_results=128):
     res = np.zeros((max_results, 5), np.float32)
     n = ctypes.c_int(0)
-    rc = load().kf_autotune(ctx, res.ctypes.data_as(_P), max_results, ctypes.byref(n), _stream(stream))
+    rc = load().kf_autotune(ctx, res.ctypes.data, max_results, ctypes.byref(n), _stream(stream))
     _check(ctx, rc, "kf_autotune")
     return res[:n.value]
 
@@ -269,7 +273,7 @@ def kf_autotune(ctx, stream=None, max_results=128):
 def kf_get_counters(ctx, stream=None):
     """The finding's counters (kf_get_counters_n, all KF_N_COUNTERS of them)."""
     c = np.zeros(KF_N_COUNTERS, np.int64)
-    _check(ctx, load().kf_get_counters_n(ctx, c.ctypes.data_as(_P), KF_N_COUNTERS, _stream(stream)),
+    _check(ctx, load().kf_get_counters_n(ctx, c.ctypes.data, KF_N_COUNTERS, _stream(stream)),
            "kf_get_counters_n")
     return dict(steps=int(c[0]), updates=int(c[1]), chi2_evals=int(c[2]), seeds=int(c[3]),
                 holes=int(c[4]), careful=int(c[5]), not_pd=int(c[6]), redone=int(c[7]),
@@ -283,7 +287,7 @@ def kf_set_stage_timing(ctx, enable=True):
 def kf_get_stage_ms(ctx, stream=None):
     """Stage durations of the last run (ms); stages that did not run are left out."""
     ms = np.zeros(6, np.float32)
-    _check(ctx, load().kf_get_stage_ms(ctx, ms.ctypes.data_as(_P), _stream(stream)), "kf_get_stage_ms")
+    _check(ctx, load().kf_get_stage_ms(ctx, ms.ctypes.data, _stream(stream)), "kf_get_stage_ms")
     names = ("bin", "find", "dedup", "fit", "adjoint", "seed_clean")
     return {k: float(v) for k, v in zip(names, ms) if v >= 0}
 
