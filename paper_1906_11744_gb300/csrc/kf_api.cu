@@ -55,7 +55,10 @@ struct kf_ctx {
   int fit_source = KF_FIT_FOUND;
   FitParams last_fit;
   DevBuf adj_align_acc, adj_align, adj_hits, adj_seed;
-  int* bad = nullptr;  // two pinned host words the load kernels report bad input to
+  // Pinned host words: two the load kernels report bad input to, one for the
+  // status word beside results written to host memory.
+  int* bad = nullptr;
+  bool host_direct = false;  // kernels reach host memory through the host's page tables
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   // What the captured graph baked in: the device address of every buffer and
@@ -130,25 +133,29 @@ cudaError_t offsets_arg(const std::vector<int>& h, void* dst, cudaStream_t st, O
   return cudaSuccess;
 }
 
-// The copies of c that come from host memory are made here and leave the list
-// (a load kernel makes those from device memory).
-cudaError_t from_host(CopyList* c, int device_ptrs, cudaStream_t st) {
-  if (device_ptrs) return cudaSuccess;
+// Host arrays of up to this many bytes in all are read and written by the copy
+// kernels themselves where the GPU shares the host's page tables: a copy
+// through the driver costs some 5 us per array, and from or to pageable memory
+// a staging pass as well (results of an 8,000-seed event 83 -> 31 us).  Larger
+// ones stay with the copy engines, which leave the SMs to a running graph.
+constexpr size_t HOST_DIRECT_BYTES = 16 << 20;
+size_t total_bytes(const CopyList& c) {
+  size_t b = 0;
+  for (int k = 0; k < c.n; ++k) b += c.bytes[k];
+  return b;
+}
+
+// The copies of c that the driver has to make from host memory are made here
+// and leave the list (a load kernel makes the others); *in_list: whether the
+// list is the kernel's.
+cudaError_t from_host(CopyList* c, int device_ptrs, bool host_direct, cudaStream_t st, bool* in_list) {
+  *in_list = device_ptrs || (host_direct && total_bytes(*c) <= HOST_DIRECT_BYTES);
+  if (*in_list) return cudaSuccess;
   for (int k = 0; k < c->n; ++k) {
     const cudaError_t e = cudaMemcpyAsync(c->dst[k], c->src[k], c->bytes[k], cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return e;
   }
   c->n = 0;
-  return cudaSuccess;
-}
-
-// Results out: to device memory in one launch, to host memory by copies.
-cudaError_t get_all(const CopyList& c, int device_ptrs, int num_sms, cudaStream_t st) {
-  if (device_ptrs) return launch_copy(c, num_sms, st);
-  for (int k = 0; k < c.n; ++k) {
-    const cudaError_t e = cudaMemcpyAsync(c.dst[k], c.src[k], c.bytes[k], cudaMemcpyDeviceToHost, st);
-    if (e != cudaSuccess) return e;
-  }
   return cudaSuccess;
 }
 
@@ -179,10 +186,8 @@ int auto_lanes(int n) {
 
 }  // namespace
 
-static int check_status(kf_ctx* ctx, cudaStream_t st) {
-  int h = 0;
-  CK(cudaMemcpyAsync(&h, ctx->status.p, sizeof(int), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
+// The error of a device status word h just read on st, which is then cleared.
+static int report_status(kf_ctx* ctx, int h, cudaStream_t st) {
   if (h == ST_OK) return KF_OK;
   CK(cudaMemsetAsync(ctx->status.p, 0, sizeof(int), st));
   CK(cudaStreamSynchronize(st));
@@ -194,6 +199,29 @@ static int check_status(kf_ctx* ctx, cudaStream_t st) {
     case ST_SEED_ROUNDS: return fail(ctx, KF_ERR_TIMEOUT, "seed cleaning: resolution did not settle");
     default: return fail(ctx, KF_ERR_CUDA, "unknown device status");
   }
+}
+static int check_status(kf_ctx* ctx, cudaStream_t st) {
+  int h = 0;
+  CK(cudaMemcpyAsync(&h, ctx->status.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+  CK(cudaStreamSynchronize(st));
+  return report_status(ctx, h, st);
+}
+// Results out: to device memory in one launch; to host memory with the status
+// word, synchronized, in one launch too or (large ones) by the driver's copies.
+static int get_all(kf_ctx* ctx, CopyList& c, int device_ptrs, cudaStream_t st) {
+  if (device_ptrs) {
+    CK(launch_copy(c, ctx->num_sms, st));
+    return KF_OK;
+  }
+  if (ctx->host_direct && total_bytes(c) <= HOST_DIRECT_BYTES) {
+    c.add(ctx->bad + 2, ctx->status.p, sizeof(int));
+    CK(launch_copy(c, ctx->num_sms, st));
+    CK(cudaStreamSynchronize(st));
+    return report_status(ctx, ctx->bad[2], st);
+  }
+  for (int k = 0; k < c.n; ++k)
+    CK(cudaMemcpyAsync(c.dst[k], c.src[k], c.bytes[k], cudaMemcpyDeviceToHost, st));
+  return check_status(ctx, st);
 }
 static int check_status_sync(kf_ctx* ctx, cudaStream_t st) { return check_status(ctx, st); }
 
@@ -337,7 +365,12 @@ int kf_create(const kf_detector* det, const kf_config* cfg, kf_ctx** out) {
     if (e == cudaSuccess) e = cudaMemcpy(ctx->eta_lut.p, lut.data(), lut.size(), cudaMemcpyHostToDevice);
   }
   if (e == cudaSuccess) e = grow(ctx->queue, 64);
-  if (e == cudaSuccess) e = cudaHostAlloc(&ctx->bad, 2 * sizeof(int), cudaHostAllocMapped);
+  if (e == cudaSuccess) e = cudaHostAlloc(&ctx->bad, 3 * sizeof(int), cudaHostAllocMapped);
+  if (e == cudaSuccess) {
+    int tables = 0;
+    e = cudaDeviceGetAttribute(&tables, cudaDevAttrPageableMemoryAccessUsesHostPageTables, dev);
+    ctx->host_direct = tables != 0;
+  }
   if (e == cudaSuccess) {
     int least = 0, greatest = 0;
     e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
@@ -429,7 +462,8 @@ int kf_load_hits(kf_ctx* ctx, int n_events, const int* ev_offsets, const float* 
   c.add(ctx->hy.p, y, sizeof(float) * n);
   c.add(ctx->hz.p, z, sizeof(float) * n);
   c.add(ctx->hlayer.p, layer, sizeof(int) * n);
-  CK(from_host(&c, device_ptrs, st));
+  bool in_list;
+  CK(from_host(&c, device_ptrs, ctx->host_direct, st, &in_list));
   OffsetArg off;
   CK(offsets_arg(ctx->hit_off_h, ctx->hit_off.p, st, &off));
   ctx->found = ctx->deduped = ctx->fitted = false;
@@ -439,7 +473,7 @@ int kf_load_hits(kf_ctx* ctx, int n_events, const int* ev_offsets, const float* 
   // Layer indices checked on the device (the caller's buffers are in use until
   // the synchronization below).
   ctx->bad[0] = 0;
-  CK(launch_load_hits(c, device_ptrs ? layer : ptr<int>(ctx->hlayer), n, ctx->g.n_surf, off, ptr<int>(ctx->hit_off),
+  CK(launch_load_hits(c, in_list ? layer : ptr<int>(ctx->hlayer), n, ctx->g.n_surf, off, ptr<int>(ctx->hit_off),
                       ctx->bad, ctx->num_sms, st));
   CK(cudaStreamSynchronize(st));
   if (ctx->bad[0]) {
@@ -514,13 +548,14 @@ int kf_load_seeds(kf_ctx* ctx, int n_events, const int* ev_offsets, const float*
   c.add(ctx->sp.p, params, sizeof(float) * 6 * (size_t)n);
   c.add(ctx->sc.p, cov, sizeof(float) * 21 * (size_t)n);
   c.add(ctx->sh.p, seed_hits, sizeof(int) * 3 * (size_t)n);
-  CK(from_host(&c, device_ptrs, st));
+  bool in_list;
+  CK(from_host(&c, device_ptrs, ctx->host_direct, st, &in_list));
   OffsetArg off;
   CK(offsets_arg(ctx->seed_off_h, ctx->seed_off.p, st, &off));
   ctx->found = ctx->deduped = ctx->fitted = false;
   // Seed hit indices checked on the device against their event's hits.
   ctx->bad[0] = ctx->bad[1] = 0;
-  CK(launch_load_seeds(c, device_ptrs ? seed_hits : ptr<int>(ctx->sh), n, n_events, off, ptr<int>(ctx->seed_off),
+  CK(launch_load_seeds(c, in_list ? seed_hits : ptr<int>(ctx->sh), n, n_events, off, ptr<int>(ctx->seed_off),
                        ptr<int>(ctx->hit_off), ptr<int>(ctx->hlayer), ctx->g.n_layers, ptr<int>(ctx->seed_event),
                        ptr<unsigned char>(ctx->keep), ctx->bad, ctx->num_sms, st));
   if (n > 0)
@@ -1006,9 +1041,7 @@ int kf_get_tracks(kf_ctx* ctx, int* hits, int* n_found, float* chi2, float* para
   c.add(params, ctx->out_p.p, sizeof(float) * 6 * n);
   c.add(cov, ctx->out_C.p, sizeof(float) * 21 * n);
   c.add(keep, ctx->keep.p, n);
-  CK(get_all(c, device_ptrs, ctx->num_sms, st));
-  if (!device_ptrs) return check_status(ctx, st);
-  return KF_OK;
+  return get_all(ctx, c, device_ptrs, st);
 }
 
 int kf_get_fit(kf_ctx* ctx, float* params, float* cov, float* chi2, int* status, int device_ptrs, void* stream) {
@@ -1021,9 +1054,7 @@ int kf_get_fit(kf_ctx* ctx, float* params, float* cov, float* chi2, int* status,
   c.add(cov, ctx->fit_C.p, sizeof(float) * 21 * n);
   c.add(chi2, ctx->fit_chi2.p, sizeof(float) * n);
   c.add(status, ctx->fit_status.p, sizeof(int) * n);
-  CK(get_all(c, device_ptrs, ctx->num_sms, st));
-  if (!device_ptrs) return check_status(ctx, st);
-  return KF_OK;
+  return get_all(ctx, c, device_ptrs, st);
 }
 
 int kf_get_counters(kf_ctx* ctx, long long* counters8, void* stream) { return kf_get_counters_n(ctx, counters8, 8, stream); }
@@ -1150,9 +1181,7 @@ int kf_get_gradient(kf_ctx* ctx, float* g_align, float* g_hits, float* g_seed, i
   c.add(g_align, ctx->adj_align.p, sizeof(float) * 2 * ctx->g.n_layers);
   c.add(g_hits, ctx->adj_hits.p, sizeof(float) * 3 * (size_t)ctx->n_hits);
   c.add(g_seed, ctx->adj_seed.p, sizeof(float) * 6 * (size_t)ctx->n_seeds);
-  CK(get_all(c, device_ptrs, ctx->num_sms, st));
-  if (!device_ptrs) return check_status(ctx, st);
-  return KF_OK;
+  return get_all(ctx, c, device_ptrs, st);
 }
 
 int kf_launch_graph(kf_ctx* ctx, void* stream) {

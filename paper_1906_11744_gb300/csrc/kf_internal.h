@@ -234,12 +234,12 @@ struct AdjParams {
 };
 
 // kf_copy.cu
-// Up to six copies of one launch.
+// Up to seven copies of one launch.
 struct CopyList {
   int n = 0;
-  void* dst[6];
-  const void* src[6];
-  size_t bytes[6];
+  void* dst[7];
+  const void* src[7];
+  size_t bytes[7];
   void add(void* d, const void* s, size_t b) {
     if (!d || b == 0) return;
     dst[n] = d;
