@@ -421,67 +421,73 @@ __global__ void k_sc_conflicts(const SeedCleanParams P, int pos_begin, int pos_e
 }
 
 // Per event (one block): the resolution rounds over the event's seeds with
-// conflicts; then the new order of its positions (kept seeds first in theta
-// order, the dropped ones from the end) and the empty outputs of the dropped
-// seeds.  Each thread splits a contiguous segment of positions; one block
-// scan of the segments' kept counts places them.
+// conflicts; then the new order of its positions: kept seeds first in theta
+// order, the dropped ones from the end.  Tiles of positions are split one
+// after the other, a ballot per warp and a scan over the warps each, so that
+// states and orders are read and written coalesced.
 __global__ void __launch_bounds__(DEDUP_THREADS) k_sc_resolve(const SeedCleanParams P, int e_begin) {
-  __shared__ int s_warp[DEDUP_THREADS / 32];
-  __shared__ int s_tot;
+  constexpr int NW = DEDUP_THREADS / 32;
+  __shared__ int s_warp[2][NW];
   const int e = e_begin + blockIdx.x;
   const int s0 = P.seed_off[e], s1 = P.seed_off[e + 1];
   if (s1 <= s0) {
     if (threadIdx.x == 0) P.kept_cnt[e] = 0;
     return;
   }
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int* list = P.list + s0;
   dd_rounds_over(Rounds{P.n_conf, P.conf, P.state, nullptr, P.status, ST_SEED_ROUNDS, P.max_rounds}, P.list_cnt[e],
                  [&](int i) { return list[i]; });
   __syncthreads();
-  const int per = (s1 - s0 + nt - 1) / nt;
-  const int a = min(s0 + tid * per, s1), b = min(a + per, s1);
-  int mine = 0;
-  for (int j = a; j < b; ++j) mine += P.state[j] == 1;
-  // exclusive scan of the kept counts over the block
-  int incl = mine;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += v;
-  }
-  if (lane == 31) s_warp[warp] = incl;
-  __syncthreads();
-  if (warp == 0) {
-    const int w = lane < nw ? s_warp[lane] : 0;
-    int wi = w;
+  int kept = 0;  // kept positions before this tile
+  for (int t0 = s0, buf = 0; t0 < s1; t0 += DEDUP_THREADS, buf ^= 1) {
+    const int j = t0 + tid;
+    const bool in = j < s1;
+    const int seed = in ? P.order[j] : 0;
+    const bool keep = in && P.state[j] == 1;
+    const unsigned b = __ballot_sync(0xffffffffu, keep);
+    if (lane == 0) s_warp[buf][warp] = __popc(b);
+    __syncthreads();  // (the other buffer is rewritten only after the next one)
+    const int w = lane < NW ? s_warp[buf][lane] : 0;
+    int incl = w;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const int v = __shfl_up_sync(0xffffffffu, wi, o);
-      if (lane >= o) wi += v;
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
     }
-    if (lane < nw) s_warp[lane] = wi - w;
-    if (lane == nw - 1) s_tot = wi;
+    const int before = __shfl_sync(0xffffffffu, incl - w, warp) + __popc(b & ((1u << lane) - 1u));
+    const int k = kept + before;  // kept positions before j
+    if (keep) P.clean_order[s0 + k] = seed;
+    else if (in) P.clean_order[s1 - 1 - (j - s0 - k)] = seed;
+    kept += __shfl_sync(0xffffffffu, incl, 31);
   }
-  __syncthreads();
-  int kr = s_warp[warp] + incl - mine;   // kept positions before this segment
-  int dr = (a - s0) - kr;                // dropped positions before it
+  if (tid == 0) P.kept_cnt[e] = kept;
+}
+
+// The empty outputs of the dropped seeds, one warp per 32 positions of the new
+// order (their scattered writes over the whole chip).
+__global__ void k_sc_dropped(const SeedCleanParams P, int pos_begin, int pos_end) {
+  const int lane = threadIdx.x & 31;
+  const int j = pos_begin + blockIdx.x * blockDim.x + threadIdx.x;
+  bool drop = false;
+  int seed = 0;
+  if (j < pos_end) {
+    const int e = P.seed_event[j];  // positions and seed indices share the event ranges
+    drop = j - P.seed_off[e] >= P.kept_cnt[e];
+    seed = P.clean_order[j];
+  }
   const size_t n = (size_t)P.ns;
-  for (int j = a; j < b; ++j) {
-    const int s = P.order[j];
-    if (P.state[j] == 1) {
-      P.clean_order[s0 + kr++] = s;
-    } else {
-      P.clean_order[s1 - 1 - dr++] = s;
+  for (unsigned m = __ballot_sync(0xffffffffu, drop); m; m &= m - 1) {
+    const int s = __shfl_sync(0xffffffffu, seed, __ffs(m) - 1);
+    for (int l = lane; l < P.L; l += 32) P.out_hits[(size_t)s * P.L + l] = -1;
+    if (lane < 21) P.out_C[lane * n + s] = P.sc[lane * n + s];
+    if (lane < 6) P.out_p[lane * n + s] = P.sp[lane * n + s];
+    if (lane == 0) {
       P.keep[s] = 0;
       P.out_n[s] = 0;
       P.out_chi2[s] = 0.f;
-      for (int l = 0; l < P.L; ++l) P.out_hits[(size_t)s * P.L + l] = -1;
-      for (int k = 0; k < 6; ++k) P.out_p[k * n + s] = P.sp[k * n + s];
-      for (int k = 0; k < 21; ++k) P.out_C[k * n + s] = P.sc[k * n + s];
     }
   }
-  if (tid == 0) P.kept_cnt[e] = s_tot;
 }
 
 }  // namespace
@@ -521,6 +527,7 @@ cudaError_t launch_seed_clean(const SeedCleanParams& P, int pos_begin, int pos_e
     k_sc_conflicts<<<blocks, threads, 0, st>>>(P, pos_begin, pos_end);
   }
   k_sc_resolve<<<n_events, DEDUP_THREADS, 0, st>>>(P, e_begin);
+  if (n > 0) k_sc_dropped<<<(n + 255) / 256, 256, 0, st>>>(P, pos_begin, pos_end);
   return cudaGetLastError();
 }
 
