@@ -83,8 +83,8 @@ struct BinParams {
   unsigned* rank;         // [n_hits]
   float4* hb;             // [n_hits]
   float4* grouped;        // [n_hits] hits grouped by (event, layer) (layer-grouped form)
-  unsigned* gtab;         // bin_group_elems(): bucket counts, bases (+ total), cursors of the
-                          // (event, layer, chunk of eta rows) buckets
+  unsigned* gtab;         // bin_group_elems(): bucket counts, bases (+ total) of the (event,
+                          // layer, chunk of eta rows) buckets
 };
 
 struct DedupParams {
