@@ -12,7 +12,9 @@ namespace kfg {
 
 namespace {
 
-constexpr int COPY_THREADS = 256;
+// Small blocks: 64 threads of these kernels find room beside a persistent finding
+// kernel of another context (its five blocks leave 4 K registers of an SM).
+constexpr int COPY_THREADS = 64;
 constexpr int COPY_UNROLL = 4;  // 16-byte words in flight per thread
 
 // bytes of src to dst by the threads (tid of nt) of the grid: 16-byte words
@@ -109,10 +111,10 @@ __global__ void __launch_bounds__(COPY_THREADS) k_find_begin(const FindBegin b) 
 }
 
 // Blocks for `bytes` of copies: enough 16-byte words in flight to reach the
-// copy bandwidth (eight blocks per SM), one word per thread below that.
+// copy bandwidth (32 blocks per SM), one word per thread below that.
 int copy_grid(size_t bytes, int num_sms) {
   const size_t want = (bytes / 16 + COPY_THREADS - 1) / COPY_THREADS;
-  return (int)std::max<size_t>(1, std::min<size_t>(want, (size_t)num_sms * 8));
+  return (int)std::max<size_t>(1, std::min<size_t>(want, (size_t)num_sms * 32));
 }
 size_t total(const CopyList& c) {
   size_t b = 0;
