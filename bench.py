@@ -61,9 +61,9 @@ WINDOW_HITS_PER_DISK_STEP = CENSUS["disks"]["window_hits_per_disk_step"]
 
 # DRAM traffic (read + write) of one k_find launch on the 100-event batch,
 # scaled by events from an ncu capture of the same kernel on 20 of its events
-# (191.46 MB: 169.83 read + 21.62 written).
+# (188.35 MB: 169.71 read + 18.64 written).
 # None whenever k_find changes until it is captured again.
-FIND_TRAFFIC_BYTES = 191.46e6 * 5
+FIND_TRAFFIC_BYTES = 188.35e6 * 5
 
 # Duplicate handling measured beside the headline step (Sec. 4.2): seed
 # cleaning on kinematics alone (eta, phi0 within 0.01, pT within 20%) and
@@ -74,13 +74,13 @@ DUP_CFG = dict(seed_clean=1, seed_deta=0.01, seed_dphi=0.01, seed_dpt=0.2, seed_
 # entry, five state values and three hit indices and writes 32 B of
 # kinematics and hits (68 B); k_sc_conflicts reads its own 32 B and writes a
 # conflict count and state (37 B; neighbours come from L2); k_sc_resolve reads
-# order and state twice, writes the new order entry and keep flag (15 B).
-CLEAN_BYTES_PER_SEED = 68 + 37 + 15
-# DRAM traffic (read + write) of the three seed-cleaning kernels per 100-event
-# batch, scaled by events from an ncu capture on 20 of its events (17.57 MB;
+# order and state, writes the new order entry and keep flag (10 B).
+CLEAN_BYTES_PER_SEED = 68 + 37 + 10
+# DRAM traffic (read + write) of the four seed-cleaning kernels per 100-event
+# batch, scaled by events from an ncu capture on 20 of its events (18.80 MB;
 # ncu flushes the caches before each kernel, so this is the cold-cache figure).
 # Set to None whenever those kernels change until they are captured again.
-CLEAN_TRAFFIC_BYTES = 17.57e6 * 5
+CLEAN_TRAFFIC_BYTES = 18.80e6 * 5
 
 FP32_LANES_PER_SM = 128
 SM_MAX_MHZ = 2070.0
