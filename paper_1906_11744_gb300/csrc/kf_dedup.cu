@@ -41,6 +41,7 @@
 // in one block over owner ranges, 33 us so (the walks 15 of them, the rounds 7).
 // Scratch (the lists, the conflict lists and the decision states) lives in
 // global memory owned by the caller.
+#include <algorithm>
 #include <mutex>
 
 #include "kf_internal.h"
@@ -106,6 +107,14 @@ __device__ __forceinline__ unsigned* dd_heads(const DedupParams& P, int t) {
   if (!P.seed_event) return P.head;  // a single event
   const int e = P.seed_event[t];
   return P.head + P.hit_off[e] + e;
+}
+
+// The list heads empty and (clear_status) the status word zero: one launch
+// instead of two memsets where a call is bound by its launches.
+__global__ void __launch_bounds__(DD_THREADS) k_dd_begin(unsigned* head, size_t n_heads, int* clear_status) {
+  const size_t i = blockIdx.x * (size_t)DD_THREADS + threadIdx.x, nt = (size_t)gridDim.x * DD_THREADS;
+  if (i == 0 && clear_status) *clear_status = ST_OK;
+  for (size_t k = i; k < n_heads; k += nt) head[k] = DD_NONE;
 }
 
 // Entry id = t L + j for hit j of track t of [t_begin, t_end).
@@ -504,13 +513,15 @@ cudaError_t launch_dedup(const DedupParams& P, int t_begin, int t_end, int e_beg
                                           clear_status ? P.status : nullptr);
     return cudaGetLastError();
   }
-  if (clear_status) {
-    const cudaError_t e = cudaMemsetAsync(P.status, 0, sizeof(int), st);
+  if (clear_status) {  // (with tracks: kf_remove_duplicates_noalloc)
+    const size_t blocks = (n_heads + DD_THREADS - 1) / DD_THREADS;
+    k_dd_begin<<<(unsigned)std::min<size_t>(std::max<size_t>(blocks, 1), 1216), DD_THREADS, 0, st>>>(
+        P.head + head_begin, n_heads, P.status);
+  } else if (n > 0) {
+    const cudaError_t e = cudaMemsetAsync(P.head + head_begin, 0xFF, sizeof(unsigned) * n_heads, st);
     if (e != cudaSuccess) return e;
   }
   if (n > 0) {
-    const cudaError_t e = cudaMemsetAsync(P.head + head_begin, 0xFF, sizeof(unsigned) * n_heads, st);
-    if (e != cudaSuccess) return e;
     const size_t entries = (size_t)n * P.L;
     k_dd_build<<<(unsigned)((entries + DD_THREADS - 1) / DD_THREADS), DD_THREADS, 0, st>>>(P, t_begin, t_end);
     constexpr int PER = DD_THREADS / DD_LANES;
