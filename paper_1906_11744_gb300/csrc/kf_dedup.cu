@@ -38,7 +38,7 @@
 // accesses to the hit table; lists need one per entry, where a table of owner
 // ranges (count, scan over all hits, fill) needed two and the scan.
 // Measured on an 8,800-track event through the allocation-free entry: 640 us
-// in one block over owner ranges, 33 us so (the walks 15 of them, the rounds 7).
+// in one block over owner ranges, 32 us so (the walks 15 of them, the rounds 7).
 // Scratch (the lists, the conflict lists and the decision states) lives in
 // global memory owned by the caller.
 #include <algorithm>
