@@ -145,18 +145,37 @@ size_t total_bytes(const CopyList& c) {
   return b;
 }
 
-// The copies of c that the driver has to make from host memory are made here
-// and leave the list (a load kernel makes the others); *in_list: whether the
-// list is the kernel's.
-cudaError_t from_host(CopyList* c, int device_ptrs, bool host_direct, cudaStream_t st, bool* in_list) {
-  *in_list = device_ptrs || (host_direct && total_bytes(*c) <= HOST_DIRECT_BYTES);
-  if (*in_list) return cudaSuccess;
+// The kernels read a caller's array as 4-byte words, which have to start on 4
+// bytes; the driver copies one that does not (a field of a packed record, a
+// view at an odd offset).
+bool on_word(const void* p) { return ((size_t)p & 3) == 0; }
+
+// The caller's arrays (c's sources) that the driver has to copy are copied here
+// and leave the list (a load kernel copies the others).
+cudaError_t load_by_driver(CopyList* c, int device_ptrs, bool host_direct, cudaStream_t st) {
+  const bool all = !device_ptrs && !(host_direct && total_bytes(*c) <= HOST_DIRECT_BYTES);
+  int kept = 0;
   for (int k = 0; k < c->n; ++k) {
-    const cudaError_t e = cudaMemcpyAsync(c->dst[k], c->src[k], c->bytes[k], cudaMemcpyHostToDevice, st);
+    if (!all && on_word(c->src[k])) {
+      c->dst[kept] = c->dst[k];
+      c->src[kept] = c->src[k];
+      c->bytes[kept++] = c->bytes[k];
+      continue;
+    }
+    const cudaError_t e = cudaMemcpyAsync(c->dst[k], c->src[k], c->bytes[k],
+                                          device_ptrs ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return e;
   }
-  c->n = 0;
+  c->n = kept;
   return cudaSuccess;
+}
+
+// Where a load kernel reads the values of the array src that it checks: in place
+// when it is on the list, else in the copy.
+const int* values_of(const CopyList& c, const int* src, const DevBuf& copy) {
+  for (int k = 0; k < c.n; ++k)
+    if (c.src[k] == src) return src;
+  return ptr<int>(copy);
 }
 
 // Copy n bytes into a device buffer from a host or device source.
@@ -462,8 +481,7 @@ int kf_load_hits(kf_ctx* ctx, int n_events, const int* ev_offsets, const float* 
   c.add(ctx->hy.p, y, sizeof(float) * n);
   c.add(ctx->hz.p, z, sizeof(float) * n);
   c.add(ctx->hlayer.p, layer, sizeof(int) * n);
-  bool in_list;
-  CK(from_host(&c, device_ptrs, ctx->host_direct, st, &in_list));
+  CK(load_by_driver(&c, device_ptrs, ctx->host_direct, st));
   OffsetArg off;
   CK(offsets_arg(ctx->hit_off_h, ctx->hit_off.p, st, &off));
   ctx->found = ctx->deduped = ctx->fitted = false;
@@ -473,7 +491,7 @@ int kf_load_hits(kf_ctx* ctx, int n_events, const int* ev_offsets, const float* 
   // Layer indices checked on the device (the caller's buffers are in use until
   // the synchronization below).
   ctx->bad[0] = 0;
-  CK(launch_load_hits(c, in_list ? layer : ptr<int>(ctx->hlayer), n, ctx->g.n_surf, off, ptr<int>(ctx->hit_off),
+  CK(launch_load_hits(c, values_of(c, layer, ctx->hlayer), n, ctx->g.n_surf, off, ptr<int>(ctx->hit_off),
                       ctx->bad, ctx->num_sms, st));
   CK(cudaStreamSynchronize(st));
   if (ctx->bad[0]) {
@@ -548,14 +566,13 @@ int kf_load_seeds(kf_ctx* ctx, int n_events, const int* ev_offsets, const float*
   c.add(ctx->sp.p, params, sizeof(float) * 6 * (size_t)n);
   c.add(ctx->sc.p, cov, sizeof(float) * 21 * (size_t)n);
   c.add(ctx->sh.p, seed_hits, sizeof(int) * 3 * (size_t)n);
-  bool in_list;
-  CK(from_host(&c, device_ptrs, ctx->host_direct, st, &in_list));
+  CK(load_by_driver(&c, device_ptrs, ctx->host_direct, st));
   OffsetArg off;
   CK(offsets_arg(ctx->seed_off_h, ctx->seed_off.p, st, &off));
   ctx->found = ctx->deduped = ctx->fitted = false;
   // Seed hit indices checked on the device against their event's hits.
   ctx->bad[0] = ctx->bad[1] = 0;
-  CK(launch_load_seeds(c, in_list ? seed_hits : ptr<int>(ctx->sh), n, n_events, off, ptr<int>(ctx->seed_off),
+  CK(launch_load_seeds(c, values_of(c, seed_hits, ctx->sh), n, n_events, off, ptr<int>(ctx->seed_off),
                        ptr<int>(ctx->hit_off), ptr<int>(ctx->hlayer), ctx->g.n_layers, ptr<int>(ctx->seed_event),
                        ptr<unsigned char>(ctx->keep), ctx->bad, ctx->num_sms, st));
   if (n > 0)
@@ -606,8 +623,9 @@ int kf_set_alignment(kf_ctx* ctx, const float* offsets, int device_ptrs, void* s
   cudaStream_t st = S(stream);
   const int L = ctx->g.n_layers;
   CK(grow(ctx->align_raw, sizeof(float) * 2 * KF_MAX_LAYERS));
-  if (offsets && !device_ptrs) CK(put(ctx->align_raw.p, offsets, sizeof(float) * 2 * L, 0, st));
-  k_align<<<1, KF_MAX_LAYERS, 0, st>>>(offsets && !device_ptrs ? ptr<float>(ctx->align_raw) : offsets, ctx->g,
+  const bool in_place = !offsets || (device_ptrs && on_word(offsets));
+  if (!in_place) CK(put(ctx->align_raw.p, offsets, sizeof(float) * 2 * L, device_ptrs, st));
+  k_align<<<1, KF_MAX_LAYERS, 0, st>>>(in_place ? offsets : ptr<float>(ctx->align_raw), ctx->g,
                                        ptr<Align4>(ctx->align4));
   CK(cudaGetLastError());
   if (!device_ptrs) CK(cudaStreamSynchronize(st));
