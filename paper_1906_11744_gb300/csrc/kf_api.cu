@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "kf_internal.h"
+#include "kf_route.h"
 
 using namespace kfg;
 
@@ -30,6 +31,7 @@ struct kf_ctx {
   bool auto_cap = false;  // block size and register budget left to the library
   int cap_blocks_per_sm = 1;  // resident blocks of the register-capped kernel
   int num_sms = 0;
+  int device = 0, n_devices = 1;
   int blocks_per_sm = 1;
   int n_events = 0, n_hits = 0, n_seeds = 0, n_seed_events = -1, max_event_hits = 0;
   std::vector<int> hit_off_h, seed_off_h;
@@ -145,29 +147,44 @@ size_t total_bytes(const CopyList& c) {
   return b;
 }
 
-// The kernels read a caller's array as 4-byte words, which have to start on 4
-// bytes; the driver copies one that does not (a field of a packed record, a
-// view at an odd offset).
-bool on_word(const void* p) { return ((size_t)p & 3) == 0; }
+// The GPU that a caller's device array lies on.  Asked for only where there is
+// more than one (about 0.3 us an array).
+int device_of(const kf_ctx* ctx, const void* p, int device_ptrs) {
+  if (!device_ptrs || ctx->n_devices < 2) return NO_DEVICE;
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return NO_DEVICE;
+  }
+  return a.type == cudaMemoryTypeDevice ? a.device : NO_DEVICE;
+}
 
-// The caller's arrays (c's sources) that the driver has to copy are copied here
-// and leave the list (a load kernel copies the others).
-cudaError_t load_by_driver(CopyList* c, int device_ptrs, bool host_direct, cudaStream_t st) {
-  const bool all = !device_ptrs && !(host_direct && total_bytes(*c) <= HOST_DIRECT_BYTES);
+// Copies by the driver of the entries k of c that no kernel takes (kernel(k)
+// false), which leave the list.
+template <class F>
+cudaError_t copy_by_driver(CopyList* c, cudaMemcpyKind kind, cudaStream_t st, F kernel) {
   int kept = 0;
   for (int k = 0; k < c->n; ++k) {
-    if (!all && on_word(c->src[k])) {
+    if (kernel(k)) {
       c->dst[kept] = c->dst[k];
       c->src[kept] = c->src[k];
       c->bytes[kept++] = c->bytes[k];
       continue;
     }
-    const cudaError_t e = cudaMemcpyAsync(c->dst[k], c->src[k], c->bytes[k],
-                                          device_ptrs ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st);
+    const cudaError_t e = cudaMemcpyAsync(c->dst[k], c->src[k], c->bytes[k], kind, st);
     if (e != cudaSuccess) return e;
   }
   c->n = kept;
   return cudaSuccess;
+}
+
+// The caller's arrays (c's sources) that the driver has to copy are copied here
+// and leave the list (a load kernel copies the others).
+cudaError_t load_by_driver(const kf_ctx* ctx, CopyList* c, int device_ptrs, cudaStream_t st) {
+  const bool direct = device_ptrs || (ctx->host_direct && total_bytes(*c) <= HOST_DIRECT_BYTES);
+  return copy_by_driver(c, device_ptrs ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st, [&](int k) {
+    return direct && kernel_reads(c->src[k], device_of(ctx, c->src[k], device_ptrs), ctx->device);
+  });
 }
 
 // Where a load kernel reads the values of the array src that it checks: in place
@@ -229,6 +246,8 @@ static int check_status(kf_ctx* ctx, cudaStream_t st) {
 // word, synchronized, in one launch too or (large ones) by the driver's copies.
 static int get_all(kf_ctx* ctx, CopyList& c, int device_ptrs, cudaStream_t st) {
   if (device_ptrs) {
+    CK(copy_by_driver(&c, cudaMemcpyDeviceToDevice, st,
+                      [&](int k) { return kernel_writes(device_of(ctx, c.dst[k], device_ptrs), ctx->device); }));
     CK(launch_copy(c, ctx->num_sms, st));
     return KF_OK;
   }
@@ -351,6 +370,8 @@ int kf_create(const kf_detector* det, const kf_config* cfg, kf_ctx** out) {
   }
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
+  ctx->device = dev;
+  if (e == cudaSuccess) e = cudaGetDeviceCount(&ctx->n_devices);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess)
     e = find_prepare(ctx->lanes, ctx->regcap, ctx->threads, ctx->g, &ctx->blocks_per_sm);
@@ -481,7 +502,7 @@ int kf_load_hits(kf_ctx* ctx, int n_events, const int* ev_offsets, const float* 
   c.add(ctx->hy.p, y, sizeof(float) * n);
   c.add(ctx->hz.p, z, sizeof(float) * n);
   c.add(ctx->hlayer.p, layer, sizeof(int) * n);
-  CK(load_by_driver(&c, device_ptrs, ctx->host_direct, st));
+  CK(load_by_driver(ctx, &c, device_ptrs, st));
   OffsetArg off;
   CK(offsets_arg(ctx->hit_off_h, ctx->hit_off.p, st, &off));
   ctx->found = ctx->deduped = ctx->fitted = false;
@@ -566,7 +587,7 @@ int kf_load_seeds(kf_ctx* ctx, int n_events, const int* ev_offsets, const float*
   c.add(ctx->sp.p, params, sizeof(float) * 6 * (size_t)n);
   c.add(ctx->sc.p, cov, sizeof(float) * 21 * (size_t)n);
   c.add(ctx->sh.p, seed_hits, sizeof(int) * 3 * (size_t)n);
-  CK(load_by_driver(&c, device_ptrs, ctx->host_direct, st));
+  CK(load_by_driver(ctx, &c, device_ptrs, st));
   OffsetArg off;
   CK(offsets_arg(ctx->seed_off_h, ctx->seed_off.p, st, &off));
   ctx->found = ctx->deduped = ctx->fitted = false;
@@ -623,7 +644,8 @@ int kf_set_alignment(kf_ctx* ctx, const float* offsets, int device_ptrs, void* s
   cudaStream_t st = S(stream);
   const int L = ctx->g.n_layers;
   CK(grow(ctx->align_raw, sizeof(float) * 2 * KF_MAX_LAYERS));
-  const bool in_place = !offsets || (device_ptrs && on_word(offsets));
+  const bool in_place =
+      !offsets || (device_ptrs && kernel_reads(offsets, device_of(ctx, offsets, device_ptrs), ctx->device));
   if (!in_place) CK(put(ctx->align_raw.p, offsets, sizeof(float) * 2 * L, device_ptrs, st));
   k_align<<<1, KF_MAX_LAYERS, 0, st>>>(in_place ? offsets : ptr<float>(ctx->align_raw), ctx->g,
                                        ptr<Align4>(ctx->align4));
