@@ -141,7 +141,9 @@ typedef struct {
   int ckpt_stride;        /* hits between forward checkpoints of the adjoint (0 = 1; 1..8) */
   int find_regcap;        /* 0 = finding kernel at the compiler's register count (blocks <= 256
                              threads); 1 = at most 102 registers, five blocks per SM (blocks
-                             <= 128 threads).  The results are identical. */
+                             <= 128 threads).  0 with block_threads = 0 leaves the choice to the
+                             library, by the size of each launch, until kf_autotune has made it.
+                             The results are identical. */
   /* Kinematic criteria (Sec. 4.2 names pT, eta and phi).  For two states A, B:
    * eta = -ln tan(theta/2); phi0 = the direction of motion at the point of the
    * helix closest to the z axis (the same for every state along a helix);

@@ -783,7 +783,9 @@ static int careful_grid(const kf_ctx* ctx, int n_seeds) {
 // candidate places than this takes the register-capped finding kernel (five
 // blocks per SM, no records of given-up seeds): its main pass is 7% faster on
 // a full chip, which from about 0.75 ms of finding on outweighs the 60 us that
-// the records save the careful pass.
+// the records save the careful pass (8 and 20 events of 8,000 seeds, N = 10:
+// 853 -> 840 and 1,884 -> 1,772 us).  With disks, whose kernels keep no
+// records, it is the faster one too (1,339 -> 1,309 and 2,999 -> 2,903 us).
 constexpr long long AUTO_CAP_CANDS = 600000;
 
 int kf_find_tracks(kf_ctx* ctx, void* stream) {
@@ -1259,11 +1261,12 @@ int kf_autotune(kf_ctx* ctx, float* results, int max_results, int* n_results, vo
   float best = 1e30f;
   int best_l = saved_lanes, best_t = saved_threads, best_p = saved_pers, best_b = saved_bps,
       best_rc = saved_rc;
-  ctx->auto_cap = false;  // the shape is the tuner's from here on
   int nr = 0;
   cudaEvent_t a, b;
   CK(cudaEventCreate(&a));
   CK(cudaEventCreate(&b));
+  const bool saved_auto = ctx->auto_cap;
+  ctx->auto_cap = false;
   int rc = KF_OK;
   for (int lanes : lane_opts) {
     if (lanes < ctx->cfg.max_cands) continue;
@@ -1317,6 +1320,7 @@ int kf_autotune(kf_ctx* ctx, float* results, int max_results, int* n_results, vo
   ctx->persistent = best_p;
   ctx->blocks_per_sm = best_b;
   ctx->regcap = best_rc;
+  ctx->auto_cap = saved_auto && !(best < 1e30f);  // a shape that was timed is the tuner's choice
   CK(find_prepare(best_l, best_rc, best_t, ctx->g, &ctx->blocks_per_sm));
   if (n_results) *n_results = nr;
   if (rc != KF_OK) return rc;
