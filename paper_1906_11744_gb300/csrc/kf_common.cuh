@@ -129,6 +129,14 @@ __device__ __forceinline__ float kmin(float a, float b) { return fminf(a, b); }
 __device__ __forceinline__ float kdiv(float a, float b) { return __fdividef(a, b); }
 __device__ __forceinline__ double kdiv(double a, double b) { return a / b; }
 __device__ __forceinline__ double kmin(double a, double b) { return fmin(a, b); }
+// ab + c for a product ab = a b that is also used by itself.  In double it is
+// stated as the fused operation, so that every function with the same formula
+// rounds alike (the fit has two forms of its double-precision step); other
+// scalars leave it to the compiler.
+template <class T>
+__device__ __forceinline__ T kprod_add(T, T, T ab, T c) { return ab + c; }
+template <>
+__device__ __forceinline__ double kprod_add<double>(double a, double b, double, double c) { return fma(a, b, c); }
 
 // sinc(psi) = sin(psi)/psi, cosc(psi) = (1 - cos psi)/psi,
 // f1 = (psi cos psi - sin psi)/psi^2, f2 = (psi sin psi - 1 + cos psi)/psi^2.
@@ -148,10 +156,10 @@ __device__ __forceinline__ void helix_fns(T psi, T& sc, T& cc, T& f1, T& f2) {
               T(0.5));
     if (sizeof(T) == 8) {  // double: extend each series by its next term
       const T q5 = q * q * q * q * q;
-      sc += q5 * T(-1.0 / 39916800.0);
-      cc += psi * q5 * T(-1.0 / 479001600.0);
-      f1 += psi * q5 * T(12.0 / 6227020800.0);
-      f2 += q5 * T(-11.0 / 479001600.0);
+      sc = kfma(q5, T(-1.0 / 39916800.0), sc);
+      cc = kfma(psi * q5, T(-1.0 / 479001600.0), cc);
+      f1 = kfma(psi * q5, T(12.0 / 6227020800.0), f1);
+      f2 = kfma(q5, T(-11.0 / 479001600.0), f2);
     }
   } else {
     T sn, cs;
@@ -160,8 +168,8 @@ __device__ __forceinline__ void helix_fns(T psi, T& sc, T& cc, T& f1, T& f2) {
     const T ip = T(1) / psi;
     sc = sn * ip;
     cc = T(2) * hs * hs * ip;
-    f1 = (cs - sc) * ip;
-    f2 = (sn - cc) * ip;
+    f1 = kprod_add(-sn, ip, -sc, cs) * ip;
+    f2 = kprod_add(T(-2) * hs * hs, ip, -cc, sn) * ip;
   }
 }
 
@@ -194,10 +202,11 @@ __device__ __forceinline__ bool path_length(T x, T y, T h, T cf, T sf, T R, T& s
   const T A = b * h;
   const T B = kfma(a, h, T(1));
   const T E = T(0.5) * h * h * dR2;
-  const T den = T(2) * B - E;
+  const T den = kprod_add(T(2), B, T(2) * B, -E);
   const T D = kfma(A, A, E * den);
   if (D < T(0)) return false;
   const T sq = ksqrt(D);
+  const T A_plus = kprod_add(b, h, A, sq), A_minus = kprod_add(b, h, A, -sq);  // A +- sq
   // Outward crossing (the usual step to the next layer): inside the cylinder
   // (E > 0), moving outward (b > 0, A = b h not zero) with den > 0, the root of
   // the sign of h is
@@ -206,15 +215,15 @@ __device__ __forceinline__ bool path_length(T x, T y, T h, T cf, T sf, T R, T& s
   // exactly this one; its quotient, arctangent and arc length are the same
   // operations as there.
   if (E > T(0) && b > T(0) && den > T(0) && A != T(0)) {
-    const T psi = T(2) * katan(kdiv(E, h > T(0) ? A + sq : A - sq));
+    const T psi = T(2) * katan(kdiv(E, h > T(0) ? A_plus : A_minus));
     s = psi * kdiv(T(1), h);
     return true;
   }
   T n0, d0, n1, d1;
   if (A >= T(0)) {
-    n0 = E; d0 = A + sq; n1 = -(A + sq); d1 = den;
+    n0 = E; d0 = A_plus; n1 = -A_plus; d1 = den;
   } else {
-    n0 = sq - A; d0 = den; n1 = E; d1 = A - sq;
+    n0 = -A_minus; d0 = den; n1 = E; d1 = A_minus;
   }
   // s_k = psi_k / h with psi_k = 2 atan(tau_k), tau_k = n_k / d_k (psi = pi for
   // d_k = 0), plus a full turn when not positive; the smaller s is taken.
@@ -244,7 +253,7 @@ __device__ __forceinline__ bool path_length(T x, T y, T h, T cf, T sf, T R, T& s
   const T dd = first ? d0 : d1, tc = first ? t0 : t1;
   const T psi = dd == T(0) ? T(3.14159265358979323846) : T(2) * katan(tc);
   T best = psi * ih;
-  if (best <= T(0)) best += turn;
+  if (best <= T(0)) best = kprod_add(psi, ih, best, turn);
   if (!(best < T(INFINITY))) return false;
   s = best;
   return true;
@@ -398,7 +407,7 @@ __device__ __forceinline__ int prop_jacobian(const T (&p)[6], T R, T kb, T z_lim
   q[1] = yn;
   q[2] = zn;
   q[3] = kap;
-  q[4] = phi + psi;
+  q[4] = kprod_add(h, s, psi, phi);
   q[5] = th;
   return 1;
 }
@@ -519,7 +528,7 @@ __device__ __forceinline__ T x0_at(const DevGeom& g, int l, T z, T* slope = null
   const int k = min((int)u, g.n_z - 2);
   const T d = (T)m[k + 1] - (T)m[k];
   if (slope) *slope = d * (T)g.z_node_inv;
-  return kfma(u - T(k), d, (T)m[k]);
+  return kfma(kprod_add(z + (T)g.z_max, (T)g.z_node_inv, u, -T(k)), d, (T)m[k]);
 }
 
 // ---------------------------------------------------------------- energy loss
@@ -661,7 +670,7 @@ __device__ __forceinline__ void add_ms(const T (&p)[6], T (&C)[21], T x0) {
   const T th0 = kdiv(T(0.0136), beta * pm) * ksqrt(t) * kfma(T(0.038), klog(t), T(1));
   const T v = th0 * th0;
   C[S6(4, 4)] += kdiv(v, sth * sth);
-  C[S6(5, 5)] += v;
+  C[S6(5, 5)] = kprod_add(th0, th0, v, C[S6(5, 5)]);
 }
 
 // ---------------------------------------------------------------- endcap disks
@@ -895,7 +904,7 @@ __device__ __forceinline__ void add_ms_disk(const T (&p)[6], T (&C)[21], T x0) {
   const T th0 = kdiv(T(0.0136), beta * pm) * ksqrt(t) * kfma(T(0.038), klog(t), T(1));
   const T v = th0 * th0;
   C[S6(4, 4)] += kdiv(v, sth * sth);
-  C[S6(5, 5)] += v;
+  C[S6(5, 5)] = kprod_add(th0, th0, v, C[S6(5, 5)]);
 }
 
 // A seed prior much looser than the hit resolution (a position variance above
