@@ -147,10 +147,12 @@ __device__ __forceinline__ void ksincos_acc(const Dir6<S>& a, Dir6<S>* s, Dir6<S
 namespace {
 
 constexpr float ADJ_CAREFUL_COS = ADJOINT_CAREFUL_COS;
-// Threads per block of the FP32 pass and of the careful pass; also the row
+// Threads per block of the FP32 pass and of the careful passes; also the row
 // stride LD (in floats) of their columns in shared memory.
 constexpr int ADJ_THREADS = 128;
 constexpr int ADJ_CAREFUL_THREADS = 32;
+// The careful passes beside an FP32 pass that fills the chip (list_wide).
+constexpr int ADJ_DBL_THREADS = 64;
 
 // Derivatives of f1 and f2 (the helix functions of kf_common.cuh) in psi:
 // f1' = -(sin psi + 2 f1)/psi, f2' = (cos psi - 2 f2)/psi, by the term-wise
@@ -1345,22 +1347,22 @@ __global__ void __launch_bounds__(ADJ_THREADS) k_adjoint(const AdjParams P) {
   adjoint_sums<ADJ_THREADS>(P, ga_all);
 }
 
-// Careful passes, one warp per block, over the tracks with double-precision
+// Careful passes, T threads per block, over the tracks with double-precision
 // steps (DBL) and over the rest of the careful list, each list dealt evenly to
 // the blocks (as k_fit_careful's: with few tracks, one per warp).  A double
 // step is bound by its unit, 64 clocks per warp instruction; a track has one
 // to three of them, and everything else of it runs in the FP32 code.  The two
 // passes are kernels of their own, beside each other: the double steps' code
-// would cost the FP32 one 96 registers.
-template <bool EL, bool DISK, bool DBL>
-__global__ void __launch_bounds__(ADJ_CAREFUL_THREADS) k_adjoint_careful(const AdjParams P) {
+// would cost the FP32 one 88 registers (255, with spills, against 167).
+template <bool EL, bool DISK, bool DBL, int T>
+__global__ void __launch_bounds__(T) k_adjoint_careful(const AdjParams P) {
   extern __shared__ float cols[];
   __shared__ float4 s_al[KF_MAX_LAYERS];
   __shared__ float s_R[KF_MAX_LAYERS];
   __shared__ double s_Ri[DBL ? KF_MAX_LAYERS : 1];
-  constexpr int T = ADJ_CAREFUL_THREADS;
   const unsigned n = DBL ? *P.dbl_count : *P.careful_count;
-  const unsigned per = min((unsigned)T, (n + gridDim.x - 1) / gridDim.x);  // tracks per warp and round
+  const unsigned spread = min(gridDim.x, (unsigned)P.careful_spread);
+  const unsigned per = min((unsigned)T, (n + spread - 1) / spread);  // tracks per warp and round
   if (blockIdx.x * per >= n) return;
   if constexpr (DBL)
     for (int l = threadIdx.x; l < P.g.n_layers; l += T) s_Ri[l] = 1.0 / (double)P.g.radius[l];
@@ -1389,22 +1391,39 @@ __global__ void k_adjoint_finish(const AdjParams P) {
 namespace {
 
 typedef void (*Kernel)(AdjParams);
+// Beside an FP32 pass that fills the chip, every block of a careful pass takes
+// the place of one of its 128-thread blocks (three of 159 registers fill an
+// SM), whatever its own size.  So from 128 tracks per SM on, the listed tracks
+// without double steps go in blocks of that size, and those with them in an
+// eighth as many blocks, of two warps (255 registers: still one such place).
+// Gradient of 176,000 / 400,000 / 800,000 tracks, ckpt_stride 1: 449 / 870 /
+// 1,453 us with one-warp blocks spread over every SM, 352 / 724 / 1,320 so;
+// stride 4: 880 / 1,630 / 2,915 and 668 / 1,448 / 2,734.  Below that size the
+// chip has room: one warp per block, over every SM.
+bool list_wide(const AdjParams& P) { return P.ns >= ADJ_THREADS * P.num_sms; }
+int pass_threads(const AdjParams& P, int pass) {
+  if (pass == ADJ_MAIN) return ADJ_THREADS;
+  if (!list_wide(P)) return ADJ_CAREFUL_THREADS;
+  return pass == ADJ_LIST ? ADJ_THREADS : ADJ_DBL_THREADS;
+}
 // The kernel of a pass for a detector (energy loss on any surface, endcap disks).
 template <bool EL, bool DISK>
-Kernel kernel_t(int pass) {
-  return pass == ADJ_MAIN ? k_adjoint<EL, DISK>
-                          : pass == ADJ_LIST ? k_adjoint_careful<EL, DISK, false> : k_adjoint_careful<EL, DISK, true>;
+Kernel kernel_t(int pass, bool wide) {
+  if (pass == ADJ_MAIN) return k_adjoint<EL, DISK>;
+  if (pass == ADJ_LIST)
+    return wide ? k_adjoint_careful<EL, DISK, false, ADJ_THREADS> : k_adjoint_careful<EL, DISK, false, ADJ_CAREFUL_THREADS>;
+  return wide ? k_adjoint_careful<EL, DISK, true, ADJ_DBL_THREADS> : k_adjoint_careful<EL, DISK, true, ADJ_CAREFUL_THREADS>;
 }
 Kernel kernel_of(const AdjParams& P, int pass) {
+  const bool wide = list_wide(P);
   bool el = P.g.n_disks > 0 && P.g.disk_eloss > 0.f;
   for (int l = 0; l < P.g.n_layers; ++l) el = el || P.g.eloss[l] > 0.f;
-  if (P.g.n_disks > 0) return el ? kernel_t<true, true>(pass) : kernel_t<false, true>(pass);
-  return el ? kernel_t<true, false>(pass) : kernel_t<false, false>(pass);
+  if (P.g.n_disks > 0) return el ? kernel_t<true, true>(pass, wide) : kernel_t<false, true>(pass, wide);
+  return el ? kernel_t<true, false>(pass, wide) : kernel_t<false, false>(pass, wide);
 }
 size_t smem_bytes(const AdjParams& P, int threads) {
   return sizeof(float) * (fp32_col_floats(P.stride) + 2 * P.g.n_layers) * (size_t)threads;
 }
-constexpr int ADJ_CAREFUL_BLOCKS = 152;  // one per SM
 
 }  // namespace
 
@@ -1419,24 +1438,20 @@ cudaError_t launch_adjoint_begin(const AdjParams& P, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   for (int pass = 0; pass < 3 && e == cudaSuccess; ++pass)
     e = cudaFuncSetAttribute((const void*)kernel_of(P, pass), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem_bytes(P, pass == ADJ_MAIN ? ADJ_THREADS : ADJ_CAREFUL_THREADS));
+                             (int)smem_bytes(P, pass_threads(P, pass)));
   return e;
 }
 
 cudaError_t launch_adjoint_pass(const AdjParams& P, int pass, cudaStream_t st) {
   if (P.ns <= 0) return cudaSuccess;
-  const Kernel k = kernel_of(P, pass);
-  if (pass == ADJ_MAIN) {
-    k<<<(P.ns + ADJ_THREADS - 1) / ADJ_THREADS, ADJ_THREADS, smem_bytes(P, ADJ_THREADS), st>>>(P);
-  } else {
-    // about a 64th of all tracks are flagged, a 350th have double steps: grids
-    // for those at 32 per block, so that a large batch packs its warps, and at
-    // least one block per SM, so that a small one spreads its tracks (of a
-    // single track each up to 10,000 tracks); striding over however many there are
-    const int of = (pass == ADJ_LIST ? 64 : 350) * ADJ_CAREFUL_THREADS;
-    const int grid = std::max(P.ns / of + 1, std::min(P.ns, ADJ_CAREFUL_BLOCKS));
-    k<<<grid, ADJ_CAREFUL_THREADS, smem_bytes(P, ADJ_CAREFUL_THREADS), st>>>(P);
+  const int threads = pass_threads(P, pass);
+  AdjParams Q = P;
+  int blocks = (P.ns + threads - 1) / threads;
+  if (pass != ADJ_MAIN) {
+    Q.careful_spread = !list_wide(P) ? P.num_sms : pass == ADJ_LIST ? 1 : std::max(1, P.num_sms / 8);
+    blocks = careful_blocks(P.ns, threads, Q.careful_spread, P.num_sms);
   }
+  kernel_of(P, pass)<<<blocks, threads, smem_bytes(P, threads), st>>>(Q);
   return cudaGetLastError();
 }
 

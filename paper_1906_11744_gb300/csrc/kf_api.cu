@@ -926,6 +926,7 @@ int kf_fit_tracks(kf_ctx* ctx, int source, const int* hit_lists, const int* n_hi
   F.ckpt_stride = ctx->cfg.ckpt_stride > 0 ? ctx->cfg.ckpt_stride : DEFAULT_CKPT_STRIDE;
   F.ckpt = nullptr;
   F.ckpt_slices = 0;
+  F.num_sms = ctx->num_sms;
   if (source == KF_FIT_FOUND) {
     if (!ctx->found) return fail(ctx, KF_ERR_STATE, "kf_fit_tracks: no found tracks");
     F.lists = ptr<int>(ctx->out_hits);
@@ -1037,6 +1038,7 @@ int kf_fit_adjoint(kf_ctx* ctx, float* g_align, float* g_hits, float* g_seed, in
   A.dbl_count = F.dbl_count;
   A.ckpt = F.ckpt;
   A.order = F.order;
+  A.num_sms = ctx->num_sms;
   stage_mark(ctx, 8, st);
   CK(launch_adjoint_begin(A, st));
   CK(fork_side(ctx, st));

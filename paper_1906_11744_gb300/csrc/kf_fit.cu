@@ -25,7 +25,6 @@ namespace {
 
 constexpr float CAREFUL_COS = 0.5f;
 constexpr int FIT_THREADS = 128;  // threads per block of the FP32 pass
-constexpr int CAREFUL_BLOCKS = 304;  // careful pass: two warps per SM
 
 // One Kalman step on an endcap disk in scalar type T (the plane, the (r-phi, r)
 // measurement, the disk's scattering and loss).
@@ -513,7 +512,8 @@ __global__ void __launch_bounds__(FIT_THREADS) k_fit(const FitParams P) {
 template <bool DISK>
 __global__ void __launch_bounds__(32) k_fit_careful(const FitParams P) {
   const unsigned n = *P.careful_count;
-  const unsigned per = min(32u, (n + gridDim.x - 1) / gridDim.x);  // tracks per warp and round
+  const unsigned spread = min(gridDim.x, (unsigned)P.careful_spread);
+  const unsigned per = min(32u, (n + spread - 1) / spread);  // tracks per warp and round
   __shared__ CoopMem mem;
   const bool whole = per == 1;  // the whole warp on one track
   if (!whole && threadIdx.x >= per) return;
@@ -558,13 +558,11 @@ cudaError_t launch_fit_main(const FitParams& P, cudaStream_t st) {
 
 cudaError_t launch_fit_careful(const FitParams& P, cudaStream_t st) {
   if (P.ns <= 0) return cudaSuccess;
-  // about a 64th of all tracks are flagged: a grid for them at 32 per block,
-  // at least CAREFUL_BLOCKS blocks (of a few tracks each in a small batch),
-  // striding over however many there are
-  const int threads = 32;
-  const int careful_blocks = std::max(P.ns / (64 * threads) + 1, std::min(P.ns, CAREFUL_BLOCKS));
-  if (P.g.n_disks > 0) k_fit_careful<true><<<careful_blocks, threads, 0, st>>>(P);
-  else k_fit_careful<false><<<careful_blocks, threads, 0, st>>>(P);
+  FitParams Q = P;
+  Q.careful_spread = 2 * P.num_sms;
+  const int blocks = careful_blocks(P.ns, 32, Q.careful_spread, P.num_sms);
+  if (P.g.n_disks > 0) k_fit_careful<true><<<blocks, 32, 0, st>>>(Q);
+  else k_fit_careful<false><<<blocks, 32, 0, st>>>(Q);
   return cudaGetLastError();
 }
 
