@@ -6,13 +6,15 @@
 // endcap disk n_eta rows in r over [disk_rmin, disk_rmax]; times n_phi bins
 // in phi = atan2(y, x).
 //
-// Layer-grouped form (grids of at most 65,536 cells per layer):
+// Layer-grouped form (grouped(): up to 16,384 phi bins and 12,288 buckets per
+// event):
 //   1. k_group_count / k_group_scan / k_group_scatter: counting sort of the
-//      hits by (event, layer, chunk of eta rows);
-//   2. k_cells: one block per (event, layer) counts its hits per cell in
+//      hits by bucket, (event, layer, chunk of eta rows of at most 16,384
+//      cells);
+//   2. k_cells: one block per bucket counts its hits per cell in
 //      shared memory (two 16-bit counters per word, padded against bank
 //      conflicts), scans the counts in place, writes the cell offsets
-//      (coalesced) and scatters its hits.  A layer of one event with more
+//      (coalesced) and scatters its hits.  A bucket with more
 //      than 65,535 hits is done by its block with global counters instead.
 // General form (larger grids): k_bin_count (key and rank of each hit by an
 // atomic count per cell), an exclusive scan of the counts (three passes),
@@ -157,8 +159,11 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(unsigned* data, siz
 }
 
 // ---- grouped form
-// Buckets: (event, layer, chunk of eta rows) with at most CHUNK_CELLS cells.
+// Buckets: (event, layer, chunk of eta rows) with at most CHUNK_CELLS cells, at
+// most GROUP_BUCKETS per event (k_group_count counts them in 48 KB of shared
+// memory).
 constexpr int CHUNK_CELLS = 16384;
+constexpr int GROUP_BUCKETS = 12288;
 constexpr int CELL_THREADS = 256;
 constexpr int CELL_HELD = 12;  // hits per thread whose cells are held in registers (3,072 per block)
 constexpr int CELL_WORDS = CHUNK_CELLS / 2;                    // two 16-bit counters per word
@@ -201,7 +206,8 @@ __device__ __forceinline__ int bucket_in_event(const BinParams& P, int i, Chunks
 // the bucket up again or counting a second time.  For 14.5 M hits the two
 // passes take 0.096 + 0.161 ms (0.058 + 0.185 with the bucket found three times
 // per hit), k_cells 0.251 (0.282 with the cell found twice); the stage of a
-// 64-event batch of 5.4 M hits 0.260 -> 0.235 ms.  A bucket index fits 16 bits: n_surf * chunks <= 64 * 256.
+// 64-event batch of 5.4 M hits 0.260 -> 0.235 ms.  A bucket index fits
+// 16 bits (GROUP_BUCKETS).
 __global__ void __launch_bounds__(GROUP_THREADS) k_group_count(const BinParams P, int e_first, int per) {
   extern __shared__ unsigned hist[];  // buckets of one event
   const Chunks ch = chunks_of(P.g.n_eta, P.g.n_phi);
@@ -424,10 +430,14 @@ size_t bin_group_elems(int n_events, int n_layers, int n_eta, int n_phi) {
   return 2 * ((size_t)n_events * n_layers * chunks_of(n_eta, n_phi).n + 1);
 }
 
+// Whether the hits are binned in the grouped form.
+static bool grouped(const BinParams& P) {
+  return P.g.n_phi <= CHUNK_CELLS && P.g.n_surf * chunks_of(P.g.n_eta, P.g.n_phi).n <= GROUP_BUCKETS && P.grouped &&
+         P.gtab;
+}
+
 size_t bin_table_elems(const BinParams& P, int n_events) {
-  return P.g.n_phi <= CHUNK_CELLS && P.grouped && P.gtab
-             ? (size_t)n_events * P.g.n_surf * chunks_of(P.g.n_eta, P.g.n_phi).n
-             : 0;
+  return grouped(P) ? (size_t)n_events * P.g.n_surf * chunks_of(P.g.n_eta, P.g.n_phi).n : 0;
 }
 
 // Bins the hits [P.h_begin, P.h_end), which must be whole events whose cells
@@ -438,7 +448,7 @@ size_t bin_table_elems(const BinParams& P, int n_events) {
 cudaError_t launch_bin(const BinParams& P, size_t bin_begin, size_t n_bins, unsigned first_pos, int max_event_hits,
                        unsigned* scan_tmp, size_t scan_tmp_elems_, cudaStream_t st) {
   const int n_hits = P.h_end - P.h_begin;
-  if (P.g.n_phi <= CHUNK_CELLS && P.grouped && P.gtab) {
+  if (grouped(P)) {
     const Chunks ch = chunks_of(P.g.n_eta, P.g.n_phi);
     const size_t per_event = (size_t)P.g.n_surf * P.g.n_eta * P.g.n_phi;
     const int e_first = (int)(bin_begin / per_event);
