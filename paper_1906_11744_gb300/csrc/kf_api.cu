@@ -553,7 +553,8 @@ int kf_load_seeds(kf_ctx* ctx, int n_events, const int* ev_offsets, const float*
   CK(grow(ctx->sfit, sizeof(float) * 29 * (size_t)n));
   CK(grow(ctx->sflag, (size_t)n));
   // records of given-up seeds: about 0.3% of them; room for a thirty-second
-  const int rec_cap = n / 32 + 64;
+  // (the disk kernels keep none)
+  const int rec_cap = ctx->g.n_disks > 0 ? 0 : n / 32 + 64;
   CK(grow(ctx->rec, sizeof(unsigned) * find_record_words(ctx->g.n_plan, ctx->g.max_cands) * (size_t)rec_cap));
   ctx->rec_cap = rec_cap;
   CK(grow(ctx->skeys, sizeof(unsigned long long) * ctx->g.max_cands * (size_t)n));

@@ -272,9 +272,10 @@ __device__ __forceinline__ Window window_disk(const FindParams& P, const float (
 // What the main pass leaves of a seed it gives up in the middle of its search,
 // at the seed's place in the list: per candidate the words below (state, chi2
 // sum, counts and flags, the task's counters), then the history's columns so
-// far.  Places at rec_cap or beyond have none (searched again from the seed).
+// far.  Places at rec_cap or beyond have none (searched again from the seed);
+// the disk kernels keep none (keeps_records).
 constexpr unsigned GIVEN_UP_RECORD = 0x80000000u;  // flag of a list entry
-constexpr int REC_CHI2 = 27, REC_META = 28, REC_IT = 29, REC_COUNT = 30, REC_HIST = 38;
+constexpr int REC_CHI2 = 27, REC_META = 28, REC_IT = 29, REC_COUNT = 30, REC_HIST = 35;
 __device__ __forceinline__ unsigned* given_up_record(const FindParams& P, int j, int HL) {
   return P.rec + (size_t)j * (REC_HIST + HL) * P.g.max_cands;
 }
@@ -779,17 +780,13 @@ __global__ void __launch_bounds__(CAP ? 128 : 256, CAP ? 5 : CAREFUL ? 1 : 2) k_
           nholes = (int)((m >> 8) & 255u);
           occ = (m >> 16) & 1u;
           finished = (m >> 17) & 1u;
-          bdone = (m >> 18) & 1u;
-          prop_done = (m >> 19) & 1u;
-          counted = (m >> 20) & 1u;
+          prop_done = (m >> 18) & 1u;
+          counted = (m >> 19) & 1u;
           c_steps = rec[(REC_COUNT + 0) * N + gl];
           c_updates = rec[(REC_COUNT + 1) * N + gl];
           c_chi2 = rec[(REC_COUNT + 2) * N + gl];
           c_holes = rec[(REC_COUNT + 3) * N + gl];
           c_npd = rec[(REC_COUNT + 4) * N + gl];
-          c_dsteps = rec[(REC_COUNT + 5) * N + gl];
-          c_dupdates = rec[(REC_COUNT + 6) * N + gl];
-          c_dholes = rec[(REC_COUNT + 7) * N + gl];
           for (int q = start; q < start + it0 - 3; ++q)
             hist[(grp * HL + q) * G + gl] = (int)rec[(REC_HIST + q) * N + gl];
         }
@@ -909,20 +906,16 @@ __global__ void __launch_bounds__(CAP ? 128 : 256, CAP ? 5 : CAREFUL ? 1 : 2) k_
           } else if (CAREFUL || !near) {
             cls = 2;
             if (!in_seed && disk) {
-              if (!RESUME || !counted) {
-                c_steps++;
-                c_dsteps++;
-              }
+              c_steps++;
+              c_dsteps++;
               DiskFrameT<float> d;
               make_frame_disk<float>(p, C, g.vr, g.vrr, d);
               const bool spd = d.f.s00 > 0.f && d.f.si00 > 0.f && d.f.si11 > 0.f;
-              if (!spd && !(RESUME && counted)) c_npd++;
+              if (!spd) c_npd++;
               const Window w = window_disk(P, p, d.f, spd);
               const unsigned* off = P.bin_off + ((size_t)ev * S + l) * ((size_t)g.n_eta * g.n_phi);
-              const unsigned c_before = c_chi2;
               scan_window<CAREFUL, true>(P, off, w, Align4{1.f, 0.f, 0.f, 0.f}, p, d.f, nfound + 1, chi2, gl, lst,
                                          cnt, c_chi2);
-              if (RESUME && counted) c_chi2 = c_before;
               after_scan();
             } else if (!in_seed) {
               if (!RESUME || !counted) c_steps++;
@@ -1249,17 +1242,13 @@ __global__ void __launch_bounds__(CAP ? 128 : 256, CAP ? 5 : CAREFUL ? 1 : 2) k_
             for (int k = 0; k < 21; ++k) rec[(6 + k) * N] = __float_as_uint(C[k]);
             rec[REC_CHI2 * N] = __float_as_uint(chi2);
             rec[REC_META * N] = (unsigned)nfound | ((unsigned)nholes << 8) | (occ ? 1u << 16 : 0u) |
-                                (finished ? 1u << 17 : 0u) | (bdone ? 1u << 18 : 0u) | (there ? 1u << 19 : 0u) |
-                                (searched ? 1u << 20 : 0u);
+                                (finished ? 1u << 17 : 0u) | (there ? 1u << 18 : 0u) | (searched ? 1u << 19 : 0u);
             rec[REC_IT * N] = (unsigned)it_up;
             rec[(REC_COUNT + 0) * N] = c_steps;
             rec[(REC_COUNT + 1) * N] = c_updates;
             rec[(REC_COUNT + 2) * N] = c_chi2;
             rec[(REC_COUNT + 3) * N] = c_holes;
             rec[(REC_COUNT + 4) * N] = c_npd;
-            rec[(REC_COUNT + 5) * N] = c_dsteps;
-            rec[(REC_COUNT + 6) * N] = c_dupdates;
-            rec[(REC_COUNT + 7) * N] = c_dholes;
             for (int q = start; q < start + it_up - 3; ++q)
               rec[(REC_HIST + q) * N] = (unsigned)hist[(grp * HL + q) * G + gl];
           }
