@@ -1421,9 +1421,10 @@ Kernel kernel_of(const AdjParams& P, int pass) {
   if (P.g.n_disks > 0) return el ? kernel_t<true, true>(pass, wide) : kernel_t<false, true>(pass, wide);
   return el ? kernel_t<true, false>(pass, wide) : kernel_t<false, false>(pass, wide);
 }
-size_t smem_bytes(const AdjParams& P, int threads) {
-  return sizeof(float) * (fp32_col_floats(P.stride) + 2 * P.g.n_layers) * (size_t)threads;
+size_t smem_bytes(int stride, int n_layers, int threads) {
+  return sizeof(float) * (fp32_col_floats(stride) + 2 * n_layers) * (size_t)threads;
 }
+size_t smem_bytes(const AdjParams& P, int threads) { return smem_bytes(P.stride, P.g.n_layers, threads); }
 
 }  // namespace
 
@@ -1436,9 +1437,11 @@ cudaError_t launch_adjoint_begin(const AdjParams& P, cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(P.g_align_acc, 0, sizeof(double) * 2 * KF_MAX_LAYERS, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(P.g_hits, 0, sizeof(float) * 3 * (size_t)P.n_hits, st);
   if (e != cudaSuccess) return e;
+  // The limit is the kernel's, shared by the contexts of every thread, so it is
+  // set to the largest of any context (201.5 KB) and not to this one's need.
   for (int pass = 0; pass < 3 && e == cudaSuccess; ++pass)
     e = cudaFuncSetAttribute((const void*)kernel_of(P, pass), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem_bytes(P, pass_threads(P, pass)));
+                             (int)smem_bytes(MAX_CKPT_STRIDE, KF_MAX_LAYERS, pass_threads(P, pass)));
   return e;
 }
 
