@@ -74,8 +74,12 @@ DUP_CFG = dict(seed_clean=1, seed_deta=0.01, seed_dphi=0.01, seed_dpt=0.2, seed_
 # entry, five state values and three hit indices and writes 32 B of
 # kinematics and hits (68 B); k_sc_conflicts reads its own 32 B and writes a
 # conflict count and state (37 B; neighbours come from L2); k_sc_resolve reads
-# order and state, writes the new order entry and keep flag (10 B).
-CLEAN_BYTES_PER_SEED = 68 + 37 + 10
+# order and state and writes the new order entry (9 B); k_sc_dropped reads every
+# position's event and seed (8 B).  Per dropped seed k_sc_dropped reads its prior
+# and writes it as the state (2 x 108 B), with its hit count, chi2, keep flag
+# (9 B) and an empty hit list (4 B per surface).
+CLEAN_BYTES_PER_SEED = 68 + 37 + 9 + 8
+CLEAN_BYTES_PER_DROPPED = 2 * 108 + 9
 # DRAM traffic (read + write) of the four seed-cleaning kernels per 100-event
 # batch, scaled by events from an ncu capture on 20 of its events (18.80 MB;
 # ncu flushes the caches before each kernel, so this is the cold-cache figure).
@@ -559,17 +563,19 @@ def main():
         dms = max_over_ranks(sum(a.elapsed_time(bb) for a, bb in zip(da, db)), dev)
         trk = td.get_tracks(stream=stream)
         clean_ms = dstage["seed_clean"] / args.steps
-        clean_gbs = n_seeds * CLEAN_BYTES_PER_SEED / (clean_ms / 1e3) / 1e9
+        n_dropped = int(n_seeds - dc["seeds"])
+        clean_bytes = n_seeds * CLEAN_BYTES_PER_SEED + n_dropped * (CLEAN_BYTES_PER_DROPPED + 4 * b.det.n_layers)
+        clean_gbs = clean_bytes / (clean_ms / 1e3) / 1e9
         hbm_peak = _measured_peak("hbm_gbs", 6800.0)
         dup = {"value": seeds_all * args.steps / (dms / 1e3), "unit": UNIT, "ms_per_step": dms / args.steps,
                "cuts": DUP_CFG, "stage_ms": {k: v / args.steps for k, v in dstage.items()},
-               "seeds_dropped_per_step": int(n_seeds - dc["seeds"]),
+               "seeds_dropped_per_step": n_dropped,
                "tracks_kept_per_step": int(trk["keep"].sum()),
                "tracks_kept_without": None,
                "gpu_launches": td.graph_kernel_count() * args.steps,
                "roofline_seed_clean": {"bound": "hbm", "achieved": clean_gbs, "peak": hbm_peak[0],
                                        "unit": "GB/s", "frac": clean_gbs / hbm_peak[0], "peak_source": hbm_peak[1],
-                                       "bytes_per_seed": CLEAN_BYTES_PER_SEED,
+                                       "bytes_per_seed": clean_bytes / n_seeds,
                                        "traffic": (CLEAN_TRAFFIC_BYTES if CLEAN_TRAFFIC_BYTES is not None
                                                    and args.config == "c4" and not args.events else None)}}
         td.close()

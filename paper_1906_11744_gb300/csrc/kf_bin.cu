@@ -173,7 +173,7 @@ constexpr int GROUP_THREADS = 256;
 // its bucket counts costs as much as some thousand hits), fewer where that
 // would leave SMs idle: 256 per block for one 2,500-track event, whose two
 // grouping passes took 20 and 36 us in 11 blocks.
-constexpr int GROUP_HITS = 4096, GROUP_BLOCKS = 304;
+constexpr int GROUP_HITS = 4096, GROUP_BLOCKS = 2 * CHIP_SMS;
 inline int group_hits(int n_hits) {
   const int per = (n_hits / GROUP_BLOCKS + GROUP_THREADS - 1) / GROUP_THREADS * GROUP_THREADS;
   return per < GROUP_THREADS ? GROUP_THREADS : per > GROUP_HITS ? GROUP_HITS : per;

@@ -12,8 +12,14 @@ namespace kfg {
 
 namespace {
 
-// Small blocks: 64 threads of these kernels find room beside a persistent finding
-// kernel of another context (its five blocks leave 4 K registers of an SM).
+// Small blocks: 64 threads of these kernels find room beside the register-capped
+// finding kernel of another context (its five blocks leave 4 K registers of an
+// SM).  The kernel at the compiler's register count, which launches of up to
+// 600,000 candidate places take, fills the register file, and a copy then waits
+// for one of its blocks: two contexts in turn take 1,098 us per step of five
+// PU-200 events (uploads, graph, downloads) where the graph alone takes 997, the
+// serial form 1,205; with copies by the driver and a finding kernel of more
+// registers it was 1,554, 1,537 and 1,806.
 constexpr int COPY_THREADS = 64;
 constexpr int COPY_UNROLL = 4;  // 16-byte words in flight per thread
 

@@ -515,7 +515,7 @@ cudaError_t launch_dedup(const DedupParams& P, int t_begin, int t_end, int e_beg
   }
   if (clear_status) {  // (with tracks: kf_remove_duplicates_noalloc)
     const size_t blocks = (n_heads + DD_THREADS - 1) / DD_THREADS;
-    k_dd_begin<<<(unsigned)std::min<size_t>(std::max<size_t>(blocks, 1), 1216), DD_THREADS, 0, st>>>(
+    k_dd_begin<<<(unsigned)std::min<size_t>(std::max<size_t>(blocks, 1), 8 * CHIP_SMS), DD_THREADS, 0, st>>>(
         P.head + head_begin, n_heads, P.status);
   } else if (n > 0) {
     const cudaError_t e = cudaMemsetAsync(P.head + head_begin, 0xFF, sizeof(unsigned) * n_heads, st);

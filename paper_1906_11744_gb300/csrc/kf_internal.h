@@ -18,6 +18,9 @@ enum : int {
   ST_SEED_ROUNDS = 5,      // seed cleaning: the resolution loop hit its iteration bound
 };
 
+// SMs of the chip, for grids of kernels that are launched without a context.
+constexpr int CHIP_SMS = 152;
+
 // Seeds of an event are taken in order of their polar angle, counting-sorted
 // into SEED_THETA_BINS equal bins of [0, pi] (the order within a bin is
 // arbitrary).
