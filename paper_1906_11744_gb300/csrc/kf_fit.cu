@@ -45,6 +45,24 @@ __device__ __forceinline__ int disk_step(const DevGeom& g, T (&p)[6], T (&C)[21]
   return KF_FIT_OK;
 }
 
+// add_ms in double with its quotients resolved: with w = |q/pT| sin(theta),
+// 0.0136/(beta p) = 0.0136 w sqrt(1 + m^2 w^2), and Var(phi) = Var(theta) /
+// sin^2(theta) without the sine.  One quotient and three roots instead of six
+// and three: a double-precision quotient takes its unit about 700 clocks.
+__device__ __forceinline__ void add_ms_double(const double (&p)[6], double (&C)[21], double x0) {
+  if (p[3] == 0.0 || x0 <= 0.0) return;
+  double sth, cth, sph, cph;
+  sincos(p[5], &sth, &cth);
+  sincos(p[4], &sph, &cph);
+  const double cd = fma(cph, p[0], sph * p[1]) * rsqrt(fma(p[0], p[0], p[1] * p[1]));
+  const double t = x0 / fabs(sth * cd);
+  const double w = fabs(p[3]) * sth;
+  const double tp = 0.0136 * fabs(p[3]) * sqrt(fma(MPION * MPION * w, w, 1.0)) * sqrt(t) * fma(0.038, log(t), 1.0);
+  const double tt = tp * sth;
+  C[S6(4, 4)] = fma(tp, tp, C[S6(4, 4)]);
+  C[S6(5, 5)] = fma(tt, tt, C[S6(5, 5)]);
+}
+
 // One Kalman step in scalar type T: propagate (unless first), update with the
 // corrected hit, scatter unless last.  Returns a KF_FIT_* status.  The fit
 // takes the library's sine and cosine throughout (ACC).
@@ -74,7 +92,8 @@ __device__ __forceinline__ int fit_step(const DevGeom& g, float (&pf)[6], float 
   chi2 += (float)chi2_of<T>(f, r0, r1);
   kf_update<T>(p, C, f, r0, r1);
   if (!last) {
-    add_ms<T, true>(p, C, x0_at<T>(g, L, p[2]));
+    if constexpr (sizeof(T) == 8) add_ms_double(p, C, x0_at<T>(g, L, p[2]));
+    else add_ms<T, true>(p, C, x0_at<T>(g, L, p[2]));
     add_eloss_ool<T, false, true>(p, C, (T)g.eloss[L]);
   }
 #pragma unroll
@@ -94,7 +113,7 @@ __device__ __forceinline__ int fit_step(const DevGeom& g, float (&pf)[6], float 
 // many lanes.  The operations and their order are fit_step's, element by
 // element (a term with a structural zero or one of J adds exactly), so that a
 // track's fit does not depend on how many others were listed.  The careful pass
-// of a 2,500-track event: 90 us in one lane per track, 70 so.
+// of a 2,500-track event: 90 us in one lane per track, 68 so.
 struct CoopMem {
   double C[36], J[36], T[36], a0[6], k0[6], k1[6], p[6];
   float f[27];
@@ -253,16 +272,14 @@ __device__ __noinline__ int fit_step_coop(const DevGeom& g, float (&pf)[6], floa
     if (pp[3] != 0.0 && x0 > 0.0) {
       sincos((lane & 1) ? pp[5] : pp[4], &sv, &cv);
       const double sph = lane_of(sv, 0), cph = lane_of(cv, 0), st = lane_of(sv, 1);
-      const double cd = fma(cph, pp[0], sph * pp[1]) * (1.0 / sqrt(fma(pp[0], pp[0], pp[1] * pp[1])));
-      // lane 0: p and beta's root, lane 1: the path's thickness and its root
-      const double quo2 = (lane & 1 ? x0 : 1.0) / (lane & 1 ? fabs(st * cd) : fabs(pp[3]) * st);
-      const double root = sqrt(lane & 1 ? quo2 : fma(quo2, quo2, MPION * MPION));
-      const double pm = lane_of(quo2, 0), t = lane_of(quo2, 1);
-      const double beta = pm / lane_of(root, 0);
-      const double th0 = 0.0136 / (beta * pm) * lane_of(root, 1) * fma(0.038, log(t), 1.0);
-      const double v44 = __dmul_rn(th0, th0) / (st * st);
-      if (lane == 18) ce += v44;  // phi, phi
-      if (lane == 20) ce = fma(th0, th0, ce);  // theta, theta
+      const double cd = fma(cph, pp[0], sph * pp[1]) * rsqrt(fma(pp[0], pp[0], pp[1] * pp[1]));
+      const double t = x0 / fabs(st * cd);
+      const double w = fabs(pp[3]) * st;
+      const double root = sqrt((lane & 1) ? t : fma(MPION * MPION * w, w, 1.0));
+      const double tp = 0.0136 * fabs(pp[3]) * lane_of(root, 0) * lane_of(root, 1) * fma(0.038, log(t), 1.0);
+      const double tt = tp * st;
+      if (lane == 18) ce = fma(tp, tp, ce);  // phi, phi
+      if (lane == 20) ce = fma(tt, tt, ce);  // theta, theta
     }
     if (g.eloss[L] > 0.f) {
       __syncwarp();
