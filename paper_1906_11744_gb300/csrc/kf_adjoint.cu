@@ -1394,13 +1394,36 @@ typedef void (*Kernel)(AdjParams);
 // Beside an FP32 pass that fills the chip, every block of a careful pass takes
 // the place of one of its 128-thread blocks (three of 159 registers fill an
 // SM), whatever its own size.  So from 128 tracks per SM on, the listed tracks
-// without double steps go in blocks of that size, and those with them in an
-// eighth as many blocks, of two warps (255 registers: still one such place).
-// Gradient of 176,000 / 400,000 / 800,000 tracks, ckpt_stride 1: 449 / 870 /
-// 1,453 us with one-warp blocks spread over every SM, 352 / 724 / 1,320 so;
-// stride 4: 880 / 1,630 / 2,915 and 668 / 1,448 / 2,734.  Below that size the
-// chip has room: one warp per block, over every SM.
+// without double steps go in blocks of that size, and those with them in blocks
+// of two warps (255 registers: still one such place), the fewer the more tracks
+// there are (dbl_spread).  Below that size the chip has room: one warp per
+// block, over every SM.
 bool list_wide(const AdjParams& P) { return P.ns >= ADJ_THREADS * P.num_sms; }
+// Blocks over which the tracks with double steps are dealt.  With few tracks the
+// call waits for their chains, which are shortest with one track per warp; with
+// many they end within the FP32 pass, whose places they take.  Both balance at
+// so many blocks as K tracks per SM and block: K is larger for the longer steps
+// onto disks, and larger where the fit's careful pass runs first on the same
+// branch, so that the FP32 pass is done before or soon after.  The adjoint (us,
+// ckpt_stride 1) with an eighth as many blocks as SMs / a quarter / half / one
+// per SM; with the rule; with all careful blocks of one warp, one per SM:
+//   gradient alone, barrel   24,000 tracks  197 / 181 / 182 / 181; 186; 188
+//                           112,000         256 / 287 / 287 / 349; 259; 353
+//                           176,000         349 / 368 / 401 / 450; 351; 454
+//                   disks    64,000         506 / 447 / 420 / 416; 410; 449
+//                           160,000         757 / 688 / 724 / 808; 716; 844
+//                           480,000       1,802 / 1,845 / 1,904 / 2,006; 1,820; 2,035
+//   after the fit,  barrel   32,000         330 / 325 / 320 / 307; 313; 312
+//                           160,000         510 / 498 / 486 / 495; 487; 501
+//                           304,000         626 / 637 / 651 / 691; 641; 728
+//                   disks    64,000         689 / 651 / 590 / 521; 520; 520
+//                           160,000         988 / 961 / 886 / 852; 877; 889
+//                           320,000       1,408 / 1,395 / 1,428 / 1,488; 1,418; 1,447
+int dbl_spread(const AdjParams& P) {
+  const long long k = (P.g.n_disks > 0 ? 300 : 100) + (P.after_fit ? 500 : 0);
+  const long long blocks = k * P.num_sms * P.num_sms / std::max(P.ns, 1);
+  return (int)std::max<long long>(std::max(1, P.num_sms / 8), std::min<long long>(P.num_sms, blocks));
+}
 int pass_threads(const AdjParams& P, int pass) {
   if (pass == ADJ_MAIN) return ADJ_THREADS;
   if (!list_wide(P)) return ADJ_CAREFUL_THREADS;
@@ -1451,7 +1474,7 @@ cudaError_t launch_adjoint_pass(const AdjParams& P, int pass, cudaStream_t st) {
   AdjParams Q = P;
   int blocks = (P.ns + threads - 1) / threads;
   if (pass != ADJ_MAIN) {
-    Q.careful_spread = !list_wide(P) ? P.num_sms : pass == ADJ_LIST ? 1 : std::max(1, P.num_sms / 8);
+    Q.careful_spread = !list_wide(P) ? P.num_sms : pass == ADJ_LIST ? 1 : dbl_spread(P);
     blocks = careful_blocks(P.ns, threads, Q.careful_spread, P.num_sms);
   }
   kernel_of(P, pass)<<<blocks, threads, smem_bytes(P, threads), st>>>(Q);

@@ -1040,6 +1040,7 @@ int kf_fit_adjoint(kf_ctx* ctx, float* g_align, float* g_hits, float* g_seed, in
   A.ckpt = F.ckpt;
   A.order = F.order;
   A.num_sms = ctx->num_sms;
+  A.after_fit = ctx->careful_fit_pending;
   stage_mark(ctx, 8, st);
   CK(launch_adjoint_begin(A, st));
   CK(fork_side(ctx, st));

@@ -253,6 +253,7 @@ struct AdjParams {
   const float* ckpt;           // the fit's checkpoints [slices][27][ns] by position
   const int* order;            // the fit's track order (position -> track)
   int num_sms;
+  bool after_fit;              // the fit's careful pass runs on the same branch before the careful passes
   int careful_spread;          // as FitParams'
 };
 
