@@ -151,8 +151,6 @@ constexpr float ADJ_CAREFUL_COS = ADJOINT_CAREFUL_COS;
 // stride LD (in floats) of their columns in shared memory.
 constexpr int ADJ_THREADS = 128;
 constexpr int ADJ_CAREFUL_THREADS = 32;
-// The careful passes beside an FP32 pass that fills the chip (list_wide).
-constexpr int ADJ_DBL_THREADS = 64;
 
 // Derivatives of f1 and f2 (the helix functions of kf_common.cuh) in psi:
 // f1' = -(sin psi + 2 f1)/psi, f2' = (cos psi - 2 f2)/psi, by the term-wise
@@ -1394,40 +1392,42 @@ typedef void (*Kernel)(AdjParams);
 // Beside an FP32 pass that fills the chip, every block of a careful pass takes
 // the place of one of its 128-thread blocks (three of 159 registers fill an
 // SM), whatever its own size.  So from 128 tracks per SM on, the listed tracks
-// without double steps go in blocks of that size, and those with them in blocks
-// of two warps (255 registers: still one such place), the fewer the more tracks
-// there are (dbl_spread).  Below that size the chip has room: one warp per
-// block, over every SM.
+// without double steps go in blocks of that size, and those with them in the
+// fewer blocks the more tracks there are (dbl_spread), of one warp: two warps
+// of 255 registers leave no room for another call's kernels.  Below that size
+// the chip has room: one warp per block, over every SM.
 bool list_wide(const AdjParams& P) { return P.ns >= ADJ_THREADS * P.num_sms; }
 // Blocks over which the tracks with double steps are dealt.  With few tracks the
 // call waits for their chains, which are shortest with one track per warp; with
-// many they end within the FP32 pass, whose places they take.  Both balance at
-// so many blocks as K tracks per SM and block: K is larger for the longer steps
-// onto disks, and larger where the fit's careful pass runs first on the same
-// branch, so that the FP32 pass is done before or soon after.  The adjoint (us,
-// ckpt_stride 1) with an eighth as many blocks as SMs / a quarter / half / one
-// per SM; with the rule; with all careful blocks of one warp, one per SM:
-//   gradient alone, barrel   24,000 tracks  197 / 181 / 182 / 181; 186; 188
-//                           112,000         256 / 287 / 287 / 349; 259; 353
-//                           176,000         349 / 368 / 401 / 450; 351; 454
-//                   disks    64,000         506 / 447 / 420 / 416; 410; 449
-//                           160,000         757 / 688 / 724 / 808; 716; 844
-//                           480,000       1,802 / 1,845 / 1,904 / 2,006; 1,820; 2,035
-//   after the fit,  barrel   32,000         330 / 325 / 320 / 307; 313; 312
-//                           160,000         510 / 498 / 486 / 495; 487; 501
-//                           304,000         626 / 637 / 651 / 691; 641; 728
-//                   disks    64,000         689 / 651 / 590 / 521; 520; 520
-//                           160,000         988 / 961 / 886 / 852; 877; 889
-//                           320,000       1,408 / 1,395 / 1,428 / 1,488; 1,418; 1,447
+// many they end within the FP32 pass, whose places they take.  So one block per
+// SM up to k tracks per SM, fewer in proportion above: k is larger for the
+// longer steps onto disks, and where the fit's careful pass runs first on the
+// same branch, so that the FP32 pass is done before or soon after.  The adjoint
+// (us, ckpt_stride 1) with a quarter as many blocks as SMs / half / one per SM;
+// with the rule; with all careful blocks of one warp, one per SM:
+//   gradient alone, barrel   24,000 tracks  185 / 185 / 184; 181; 189
+//                           176,000         370 / 400 / 450; 350; 454
+//                           400,000         742 / 790 / 840; 705; 859
+//                           800,000       1,330 / 1,330 / 1,351; 1,323; 1,447
+//                   disks   160,000         687 / 724 / 808; 751; 844
+//   after the fit,  barrel   32,000         324 / 323 / 307; 311; 312
+//                           160,000         506 / 495 / 495; 490; 501
+//                           800,000       1,378 / 1,389 / 1,413; 1,380; 1,512
+//                   disks    32,000         365 / 296 / 295; 290; 296
+//                            64,000         652 / 604 / 521; 526; 520
+//                           160,000         965 / 917 / 852; 864; 889
+//                           400,000       1,640 / 1,671 / 1,726; 1,662; 1,716
+// Calls in a row, whose loads and finding run beside the adjoint before them,
+// want fewer blocks: 20 events with disks 3,487 / 3,523 / 3,541; 3,541; 3,560 us
+// a call, 4,092 / 4,051 / 4,055; 4,055; 4,060 waited for one by one.
 int dbl_spread(const AdjParams& P) {
-  const long long k = (P.g.n_disks > 0 ? 300 : 100) + (P.after_fit ? 500 : 0);
+  const long long k = P.g.n_disks > 0 ? (P.after_fit ? 1100 : 300) : (P.after_fit ? 600 : 100);
   const long long blocks = k * P.num_sms * P.num_sms / std::max(P.ns, 1);
   return (int)std::max<long long>(std::max(1, P.num_sms / 8), std::min<long long>(P.num_sms, blocks));
 }
 int pass_threads(const AdjParams& P, int pass) {
   if (pass == ADJ_MAIN) return ADJ_THREADS;
-  if (!list_wide(P)) return ADJ_CAREFUL_THREADS;
-  return pass == ADJ_LIST ? ADJ_THREADS : ADJ_DBL_THREADS;
+  return pass == ADJ_LIST && list_wide(P) ? ADJ_THREADS : ADJ_CAREFUL_THREADS;
 }
 // The kernel of a pass for a detector (energy loss on any surface, endcap disks).
 template <bool EL, bool DISK>
@@ -1435,7 +1435,7 @@ Kernel kernel_t(int pass, bool wide) {
   if (pass == ADJ_MAIN) return k_adjoint<EL, DISK>;
   if (pass == ADJ_LIST)
     return wide ? k_adjoint_careful<EL, DISK, false, ADJ_THREADS> : k_adjoint_careful<EL, DISK, false, ADJ_CAREFUL_THREADS>;
-  return wide ? k_adjoint_careful<EL, DISK, true, ADJ_DBL_THREADS> : k_adjoint_careful<EL, DISK, true, ADJ_CAREFUL_THREADS>;
+  return k_adjoint_careful<EL, DISK, true, ADJ_CAREFUL_THREADS>;
 }
 Kernel kernel_of(const AdjParams& P, int pass) {
   const bool wide = list_wide(P);
